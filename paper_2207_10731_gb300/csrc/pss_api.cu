@@ -438,7 +438,9 @@ pss_status ensure_sorted(pss_handle* h, int64_t nnz, cudaStream_t st) {
         const size_t n = (size_t)(npairs > 0 ? npairs : 1);
         PSS_TRY(cudaMallocAsync(&h->sb.pair_x, sizeof(uint32_t) * n, st));
         PSS_TRY(cudaMallocAsync(&h->sb.sorted_e, sizeof(unsigned long long) * n, st));
-        PSS_TRY(cudaMallocAsync(&h->sb.bnd, sizeof(float) * 64 * (size_t)window_records((int64_t)n),
+        PSS_TRY(cudaMallocAsync(&h->sb.bnd,
+                                sizeof(float) * 64 *
+                                    (size_t)window_records((int64_t)n, h->sm_count),
                                 st));
         PSS_TRY(cudaMallocAsync(&h->sb.segn, sizeof(uint32_t) * (size_t)local_segments((int64_t)n),
                                 st));
@@ -868,6 +870,9 @@ static pss_status copy_stats(pss_handle* h, cudaStream_t st) {
     return PSS_OK;
 }
 
+// Bags of several ids: the sorted path reads a bag's gradient row once per id.
+static bool rows_reread(const pss_handle* h) { return h->last_nnz > h->dp.T * h->last_B; }
+
 // Sorted path with the window reduce: sort (with `touch`, also list the
 // touched blocks), then every element's gradient stored once into gexp
 // (fp32, zero on entry).
@@ -881,7 +886,8 @@ static pss_status sorted_window(pss_handle* h, const float* dgrad, bool staged, 
     {
         LaunchScope ls(h, PSS_K_REDUCE, st, 2);
         const WindowSink ws{gexp, h->sb.bnd};
-        PSS_TRY(launch_window_reduce(h->sb, npairs, dgrad, h->dp, ws, h->sm_count, st));
+        PSS_TRY(launch_window_reduce(h->sb, npairs, dgrad, h->dp, ws, rows_reread(h),
+                                     h->sm_count, st));
     }
     return copy_stats(h, st);
 }
@@ -927,7 +933,7 @@ static pss_status sorted_into64(pss_handle* h, const float* dgrad, bool staged, 
     {
         LaunchScope ls(h, PSS_K_REDUCE, st);
         PSS_TRY(launch_sorted_reduce(h->sb, npairs, dgrad, h->dp, h->g64, local,
-                                     !local && use_radix(h), h->sm_count, st));
+                                     !local && use_radix(h), rows_reread(h), h->sm_count, st));
     }
     return local ? PSS_OK : copy_stats(h, st);
 }

@@ -212,21 +212,21 @@ __device__ __forceinline__ void split_slot(int64_t s, int64_t B, uint64_t Binv, 
 // keep their sign and fraction.
 __device__ __forceinline__ double widen(float f) {
     const uint32_t u = __float_as_uint(f);
+    // normal numbers (exponent field 1 .. 254) in four instructions: the
+    // arithmetic shift moves the exponent and the top 20 fraction bits into
+    // the high word, and the mask drops the two copies of the sign it leaves
+    if (((u + 0x00800000u) & 0x7fffffffu) >= 0x01000000u)
+        return __hiloint2double((((int)u >> 3) & (int)0x8fffffffu) + (896 << 20), (int)(u << 29));
     const uint64_t sign = (uint64_t)(u & 0x80000000u) << 32;
-    const uint32_t e = (u >> 23) & 0xffu;
     const uint32_t m = u & 0x7fffffu;
-    uint64_t bits;
-    if (e == 0xffu) {
-        bits = sign | (uint64_t(0x7ff) << 52) | ((uint64_t)m << 29);
-    } else if (e != 0u) {
-        bits = sign | ((uint64_t)(e + 896u) << 52) | ((uint64_t)m << 29);
-    } else if (m == 0u) {
-        bits = sign;
-    } else {
-        // m * 2^-149 with the leading one at bit p: exponent p - 149
+    uint64_t bits = sign;                                        // zeros
+    if ((u & 0x7f800000u) != 0u) {                               // infinities, NaNs
+        bits |= (uint64_t(0x7ff) << 52) | ((uint64_t)m << 29);
+    } else if (m != 0u) {
+        // subnormal: m * 2^-149 with the leading one at bit p, exponent p - 149
         const int p = 31 - __clz(m);
-        bits = sign | ((uint64_t)(p + 874) << 52) |
-               (((uint64_t)m << (52 - p)) & ((uint64_t(1) << 52) - 1));
+        bits |= ((uint64_t)(p + 874) << 52) |
+                (((uint64_t)m << (52 - p)) & ((uint64_t(1) << 52) - 1));
     }
     return __longlong_as_double((long long)bits);
 }

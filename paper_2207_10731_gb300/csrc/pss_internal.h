@@ -84,7 +84,7 @@ struct SortedBuffers {
     uint32_t* q_row;              // nnz output rows b*T + t written by the forward
     unsigned long long* sorted_e; // nnz*J entries (x << 32 | row*J + j), grouped by x
     unsigned long long* stats;    // [0] valid pairs, [1] distinct buckets
-    float* bnd;                   // window reduce: boundary records, 64 floats per task
+    float* bnd;                   // window reduce: boundary records, 64 floats per range
     uint32_t* segn;               // local sort: valid pairs of each segment
     // counting sort (R <= kCountSortMaxR)
     uint32_t* ccnt;               // R counts per bucket (zero between sorts)
@@ -129,10 +129,11 @@ cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, ui
 // Reduce of the sorted entries into g (fp64).  `local`: the entries come from
 // the segment-local sort (one run per bucket and segment).  `count_runs`: the
 // reduce counts the distinct buckets into stats[1] (the radix sort's entries;
-// the counting sort's scan counts them itself).
+// the counting sort's scan counts them itself).  `reread`: the gradient's rows
+// are read several times (bags of several ids), so they are kept in L2.
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
-                                 int sm_count, cudaStream_t st);
+                                 bool reread, int sm_count, cudaStream_t st);
 // Window reduce (see pss_sorted.cu): run sums go into each task's sliding
 // element window; every element's gradient is stored once into gexp (fp32,
 // zero where the batch adds nothing; the caller zero-fills it), in a fixed
@@ -141,13 +142,14 @@ cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const 
 // wrap.
 struct WindowSink {
     float* gexp;    // gradient out, M elements
-    float* bnd;     // window_records(npairs) records of 64 floats
+    float* bnd;     // window_records records of 64 floats
 };
 bool window_reduce_ok(const DevParams& p, const float* gout);
-int64_t window_records(int64_t npairs);
+// Boundary records for any batch of up to npairs pairs.
+int64_t window_records(int64_t npairs, int sm_count);
 cudaError_t launch_window_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
-                                 const DevParams& p, const WindowSink& ws, int sm_count,
-                                 cudaStream_t st);
+                                 const DevParams& p, const WindowSink& ws, bool reread,
+                                 int sm_count, cudaStream_t st);
 
 // Kernel launchers (return the CUDA launch error).  `grid_cap` bounds the
 // grid of grid-stride kernels; 0 lets the launcher decide.

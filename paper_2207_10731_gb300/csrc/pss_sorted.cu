@@ -1046,33 +1046,41 @@ k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
     if (count_runs && lane == 0 && nstart) atomicAdd(stats + 1, (unsigned long long)nstart);
 }
 
-// Reduce for 32-element chunks that tile the rows (Z = 32 dividing d): the
-// upstream-gradient chunks of a warp's task are staged asynchronously into
-// shared memory (cp.async, 16 bytes per lane), kAD - 1 stages of kAS chunks in
-// flight per warp, so the data in flight is bounded by shared memory rather
-// than registers.  Lane z then sums element z of each chunk (compensated; a
-// stage that continues the current run is summed as a tree first) and adds
-// every run's sum once into the fp64 accumulator.
+// Reduce for 32-element chunks that tile the rows (Z = 32 dividing d).  Each
+// warp owns one contiguous range of `per` sorted entries (a multiple of 32; the
+// ranges of neighbouring warps go to different CTAs, so that every SM gets
+// entries from all over the batch) and walks it in blocks of 32 entries, one
+// entry per lane: the block's run boundaries are one ballot, and the chunks'
+// row numbers reach the copying lanes by shuffles.  The chunks are staged into
+// shared memory with cp.async (16 bytes per lane, 4 chunks per instruction) in
+// stages of kAS chunks, kAD - 1 stages in flight without a break from block to
+// block.  Lane z then sums element z of each chunk (compensated; a stage that
+// continues the current run is summed as a tree first) and adds every run's
+// sum once.
+// What bounds it: instruction issue where runs are short or the gradient is
+// re-read from L2 (one 128-byte load, its addition and the run's flush per
+// entry), random 128-byte HBM reads otherwise.
 constexpr int kAS = 8;          // chunks per stage
 constexpr int kAD = 4;          // ring slots (kAD - 1 stages in flight)
-// sorted entries per task.  Measured: 256 gave the multi-hot reduce 0.254
-// against 0.268 ms and left the Criteo-TB one unchanged, but its 48 KB of
-// shared memory allow one CTA less per SM and a batch of 16384 leaves ~1.4
-// tasks per warp: that reduce took 77 against 57 us.
-constexpr int kAPiece = 128;
+static_assert(kAS * kAD == 32, "a block of 32 entries fills the ring once");
+constexpr int kAMinPer = 64;    // entries per warp at least
 
-// L2 policy for data read once (the upstream gradient, the sorted entries):
-// evicted first, so that the streams do not push the fp64 accumulator and the
-// shared array out of L2.
+// L2 policies: entries, and a gradient whose rows are read once, are evicted
+// first, so that the streams do not push the fp64 accumulator and the shared
+// array out of L2; a gradient whose rows are read again stays.
 __device__ __forceinline__ uint64_t l2_evict_first() {
     uint64_t pol;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem, uint64_t pol) {
-    const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+__device__ __forceinline__ uint64_t l2_evict_normal() {
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ void cp_async16(uint32_t smem, const void* gmem, uint64_t pol) {
     asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;\n"
-                 :: "r"(sa), "l"(gmem), "l"(pol) : "memory");
+                 :: "r"(smem), "l"(gmem), "l"(pol) : "memory");
 }
 __device__ __forceinline__ unsigned long long ld_once_u64(const unsigned long long* p,
                                                           uint64_t pol) {
@@ -1090,51 +1098,102 @@ __device__ __forceinline__ void cp_async_wait() {
 
 // Where the staged reduce puts each run's sum (SINK):
 //   kSinkF64   added into the fp64 gradient accumulator g (red.global.add.f64);
-//   kSinkOnce  added into the task's ELEMENT WINDOW: the runs of a task come in
+//   kSinkOnce  added into the range's ELEMENT WINDOW: the runs of a range come in
 //              ascending bucket order, so the 32 elements [wb, wb + 32) that
 //              lane z holds (element wb + z) slide forward; an element that
-//              leaves the window has all of the task's contributions.  If no
-//              other task can add to it (no bucket of the task before or after
+//              leaves the window has all of the range's contributions.  If no
+//              other range can add to it (no bucket of the range before or after
 //              this one reaches it), its gradient is final and is stored once
 //              into ws.gexp (fp32).  Otherwise its partial sum goes to the
-//              task's boundary record (bnd[task][0..32): the window of its
+//              range's boundary record (bnd[range][0..32): the window of its
 //              first bucket, [32..64): of its last), and k_window_combine
 //              stores it.  Every element's additions then happen in a fixed
 //              order, and nothing is added atomically.
 constexpr int kSinkF64 = 0;
 constexpr int kSinkOnce = 1;
 
-template <int SINK>
+// LOCAL: the segment-local layout (k_sort_local): segment s holds segn[s] valid
+// entries from s*kLS on; otherwise one sorted run of stats[0] valid entries.
+template <int SINK, bool LOCAL, bool SG>
 __global__ void __launch_bounds__(kThreads, 4)
 k_async_reduce(const unsigned long long* __restrict__ sorted_e,
-               unsigned long long* __restrict__ stats, int64_t npairs,
-               const float* __restrict__ gout, int64_t G, uint32_t smask,
-               double* __restrict__ g, WindowSink ws, const uint32_t* __restrict__ segn,
-               bool count_runs) {
+               unsigned long long* __restrict__ stats, int64_t npairs, int64_t per,
+               const float* __restrict__ gout, bool reread, uint32_t G, double* __restrict__ g,
+               WindowSink ws, const uint32_t* __restrict__ segn, bool count_runs) {
     pdl_prologue();
     __shared__ __align__(16) float s_ring[kWarps][kAD][kAS][32];
-    __shared__ unsigned long long s_ent[kWarps][kAPiece];
-    // segn: the segment-local layout (k_sort_local), kLS / kAPiece tasks per
-    // segment, each cut at the segment's valid entries; otherwise one sorted
-    // run of stats[0] valid entries
-    constexpr int kPieces = kLS / kAPiece;
-    const bool local = segn != nullptr;
     const int64_t total =
-        local ? npairs : (int64_t)(stats[0] < (unsigned long long)npairs ? stats[0] : npairs);
-    const int64_t ntasks =
-        local ? ((npairs + kLS - 1) / kLS) * kPieces : (total + kAPiece - 1) / kAPiece;
+        LOCAL ? ((npairs + kLS - 1) / kLS) * kLS
+              : (int64_t)(stats[0] < (unsigned long long)npairs ? stats[0] : npairs);
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    unsigned long long* ent = s_ent[warp];
-    const int64_t wstride = (int64_t)gridDim.x * kWarps;
+    const int64_t task = (int64_t)warp * gridDim.x + blockIdx.x;
+    const int64_t e0 = task * per;
+    if (e0 >= total) return;
+    const int64_t e1 = (e0 + per < total) ? e0 + per : total;
+    const int nblk = (int)((e1 - e0 + 31) >> 5);
+    const uint64_t pol_once = l2_evict_first();
+    const uint64_t pol = reread ? l2_evict_normal() : pol_once;
+    const float* gl = gout + (lane & 7) * 4;      // this lane's 16 bytes of a chunk
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(
+        &s_ring[warp][0][lane >> 3][(lane & 7) * 4]);
+    const float* buf = &s_ring[warp][0][0][lane];
     constexpr unsigned long long kNone = (unsigned long long)kBad << 32;
-    const uint64_t pol = l2_evict_first();
+
+    // entry `lane` of block k: bucket in the high word, chunk number (and sign)
+    // in the low one; past the range (or a segment's valid entries): kNone,
+    // whose chunk 0 is read but never added
+    auto load_block = [&](int k) -> unsigned long long {
+        const int64_t e = e0 + (int64_t)k * 32 + lane;
+        if (LOCAL) {
+            if (k >= nblk) return kNone;
+            const uint32_t n = __ldg(segn + (e >> kLSLog2));
+            return ((uint32_t)e & (uint32_t)(kLS - 1)) < n ? ld_once_u64(sorted_e + e, pol_once)
+                                                           : kNone;
+        }
+        return e < e1 ? ld_once_u64(sorted_e + e, pol_once) : kNone;
+    };
+    // copy stage s of the block whose low words are r into ring slot s
+    auto issue = [&](uint32_t r, int s) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t rr = __shfl_sync(0xffffffffu, r, s * kAS + h * 4 + (lane >> 3));
+            cp_async16(ring + (uint32_t)(s * kAS + h * 4) * 128u,
+                       gl + (uint64_t)(SG ? rr & 0x7fffffffu : rr) * 32u, pol);
+        }
+    };
+
+    unsigned long long ent = load_block(0);
+    uint32_t x0 = (uint32_t)(ent >> 32), r0 = (uint32_t)ent;   // block k
+    ent = load_block(1);
+    uint32_t x1 = (uint32_t)(ent >> 32), r1 = (uint32_t)ent;   // block k + 1
+#pragma unroll
+    for (int s = 0; s < kAD - 1; ++s) {
+        issue(r0, s);
+        cp_async_commit();
+    }
+    uint32_t cur = __shfl_sync(0xffffffffu, x0, 0);            // bucket of the open run
+    uint32_t xlast = cur;                                      // last bucket of the block before
+    uint32_t nstart = 0;   // distinct buckets: entries whose bucket differs from the one before
     float sum = 0.f, comp = 0.f;
-    // window sink: lane z holds element wb + z; the task's head boundary ends
+    // the entry before the range: the window's head boundary, and whether the
+    // range's first bucket counts as distinct
+    uint32_t xprev = kBad;
+    if (!LOCAL && e0 > 0 && (SINK != kSinkF64 || count_runs))
+        xprev = (uint32_t)(__ldg(sorted_e + e0 - 1) >> 32);
+    if (xprev != cur) nstart = 1;
+    // window sink: lane z holds element wb + z; the range's head boundary ends
     // at hb_end, its tail boundary starts at tb_start; hx and tx are the first
     // elements of its first and last buckets
-    int64_t wb = 0, hb_end = 0, tb_start = 0, hx = 0, tx = 0, task = 0;
+    int64_t wb = 0, hb_end = 0, tb_start = 0, hx = 0, tx = 0;
     float acc = 0.f, accc = 0.f;
+    if (SINK != kSinkF64) {
+        hx = (int64_t)cur * G;
+        tx = (int64_t)(uint32_t)(__ldg(sorted_e + e1 - 1) >> 32) * G;
+        hb_end = (e0 > 0) ? (int64_t)xprev * G + 32 : 0;
+        tb_start = (e1 < total) ? (int64_t)(uint32_t)(__ldg(sorted_e + e1) >> 32) * G : INT64_MAX;
+        wb = hx;
+    }
     auto finalize = [&](int lim) {   // the window's first lim elements are done
         if (lane < lim) {
             const int64_t e = wb + lane;
@@ -1148,137 +1207,91 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
             }
         }
     };
-    auto flush = [&](uint32_t x) {
-        if (SINK == kSinkF64) {
-            if (sum != 0.f) red_add_f64(g + (int64_t)x * G + lane, widen(sum));
-        } else {
-            const int64_t xb = (int64_t)x * G;
-            const int64_t sh = xb - wb;           // >= 0: buckets ascend
-            if (sh > 0) {
-                finalize(sh < 32 ? (int)sh : 32);
-                if (sh >= 32) {
-                    acc = accc = 0.f;
-                } else {
-                    const float a2 = __shfl_down_sync(0xffffffffu, acc, (int)sh);
-                    const float c2 = __shfl_down_sync(0xffffffffu, accc, (int)sh);
-                    const bool in = lane + (int)sh < 32;
-                    acc = in ? a2 : 0.f;
-                    accc = in ? c2 : 0.f;
+    double* const glane = g + lane;
+    auto flush = [&]() {
+        if (cur != kBad) {
+            if (SINK == kSinkF64) {
+                red_add_f64(glane + (uint64_t)cur * G, widen(sum));
+            } else {
+                const int64_t xb = (int64_t)cur * G;
+                const int64_t sh = xb - wb;           // >= 0: buckets ascend
+                if (sh > 0) {
+                    finalize(sh < 32 ? (int)sh : 32);
+                    if (sh >= 32) {
+                        acc = accc = 0.f;
+                    } else {
+                        const float a2 = __shfl_down_sync(0xffffffffu, acc, (int)sh);
+                        const float c2 = __shfl_down_sync(0xffffffffu, accc, (int)sh);
+                        const bool in = lane + (int)sh < 32;
+                        acc = in ? a2 : 0.f;
+                        accc = in ? c2 : 0.f;
+                    }
+                    wb = xb;
                 }
-                wb = xb;
+                kahan_add(acc, accc, sum - comp);
             }
-            kahan_add(acc, accc, sum - comp);
         }
         sum = comp = 0.f;
     };
-    uint32_t nstart = 0;   // distinct buckets: entries whose bucket differs from the one before
-    for (int64_t t = (int64_t)blockIdx.x * kWarps + warp; t < ntasks; t += wstride) {
-        int64_t e0;
-        int n;
-        if (local) {
-            const int64_t s = t / kPieces;
-            const int k = (int)(t - s * kPieces);
-            const int left = (int)__ldg(segn + s) - k * kAPiece;
-            if (left <= 0) continue;
-            e0 = s * kLS + (int64_t)k * kAPiece;
-            n = left < kAPiece ? left : kAPiece;
-        } else {
-            e0 = t * kAPiece;
-            n = (int)((e0 + kAPiece < total) ? kAPiece : total - e0);
-        }
-#pragma unroll
-        for (int h = 0; h < kAPiece; h += 32)
-            ent[h + lane] = (h + lane < n) ? ld_once_u64(sorted_e + e0 + h + lane, pol) : kNone;
-        __syncwarp();
-        const int nst = (n + kAS - 1) / kAS;
-        // copy stage st (kAS chunks of 128 bytes = 64 pieces of 16 bytes)
-        auto issue = [&](int st) {
-            if (st < nst) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int pc = lane + 32 * h;
-                    const int i = pc >> 3;
-                    const int part = pc & 7;
-                    const int e = st * kAS + i;
-                    if (e < n) {
-                        const uint32_t r =
-                            reinterpret_cast<const uint32_t*>(ent)[2 * e] & ~smask;  // low word
-                        cp_async16(&s_ring[warp][st % kAD][i][part * 4],
-                                   gout + (uint64_t)r * 32u + (uint32_t)(part * 4), pol);
-                    }
-                }
-            }
+
+    for (int k = 0; k < nblk; ++k) {
+        const unsigned long long e2 = load_block(k + 2);   // in flight during block k
+        // bit i: entry i starts a run
+        uint32_t xp = __shfl_up_sync(0xffffffffu, x0, 1);
+        if (lane == 0) xp = xlast;
+        const uint32_t heads = __ballot_sync(0xffffffffu, x0 != xp);
+        xlast = __shfl_sync(0xffffffffu, x0, 31);
+        if (!LOCAL && count_runs)
+            nstart += __popc(heads & __ballot_sync(0xffffffffu, x0 != kBad));
+        const uint32_t signs = SG ? __ballot_sync(0xffffffffu, (int32_t)r0 < 0) : 0u;
+        // the window sink keeps one copy of the stage: unrolled four times, its
+        // flushes outgrow the instruction cache (batch 20011 of the Criteo-TB
+        // shape: 116 us against 80); the fp64 sink gains from the unrolling
+        // (multi-hot shape: 200 us against 232)
+        constexpr int kUnroll = SINK == kSinkF64 ? kAD : 1;
+#pragma unroll kUnroll
+        for (int s = 0; s < kAD; ++s) {
+            cp_async_wait<kAD - 2>();
+            __syncwarp();   // stage s is in, and every lane has read the slot filled next
+            if (s == 0 || k + 1 < nblk) issue(s == 0 ? r0 : r1, (s + kAD - 1) & (kAD - 1));
             cp_async_commit();
-        };
-#pragma unroll
-        for (int st = 0; st < kAD - 1; ++st) issue(st);
-        sum = comp = 0.f;
-        uint32_t cur = (uint32_t)(ent[0] >> 32);
-        // the previous entry's bucket: the window's head boundary, and the count
-        // of distinct buckets when this pass makes it
-        const bool need_prev = (SINK != kSinkF64) || count_runs;
-        const uint32_t xprev = (e0 > 0 && !local && need_prev)
-                                   ? (uint32_t)(__ldg(sorted_e + e0 - 1) >> 32)
-                                   : kBad;
-        nstart += (e0 == 0 || xprev != cur) ? 1u : 0u;
-        if (SINK != kSinkF64) {
-            task = t;
-            hx = (int64_t)cur * G;
-            tx = (int64_t)(uint32_t)(ent[n - 1] >> 32) * G;
-            hb_end = (e0 > 0) ? (int64_t)xprev * G + 32 : 0;
-            tb_start = (e0 + n < total) ? (int64_t)(uint32_t)(__ldg(sorted_e + e0 + n) >> 32) * G
-                                        : INT64_MAX;
-            wb = hx;
-            acc = accc = 0.f;
-        }
-        for (int st = 0; st < nst; ++st) {
-            issue(st + kAD - 1);
-            cp_async_wait<kAD - 1>();
-            __syncwarp();
-            const float* buf = &s_ring[warp][st % kAD][0][0];
-            const uint32_t* ex = reinterpret_cast<const uint32_t*>(ent + st * kAS) + 1;  // high words: x
-            // the entries are sorted and padded with kBad: when the stage's last
-            // bucket continues the run, the stage is full and all of it does
             // all loads first, in one round trip (the flush's reduction is a
-            // memory barrier for the compiler, so later loads would not overlap);
-            // chunks past the task's end are never read as values
-            const uint32_t xlast = ex[2 * (kAS - 1)];
+            // memory barrier for the compiler, so later loads would not overlap)
             float v[kAS];
 #pragma unroll
-            for (int i = 0; i < kAS; ++i) v[i] = buf[i * 32 + lane];
-            if (smask) {
-                // signed hashing: each entry's sign is bit 31 of its low word
+            for (int i = 0; i < kAS; ++i) v[i] = buf[(s * kAS + i) * 32];
+            if (SG) {
 #pragma unroll
-                for (int i = 0; i < kAS; ++i) v[i] = sign_by(v[i], ex[2 * i - 1] & smask);
+                for (int i = 0; i < kAS; ++i)
+                    v[i] = sign_by(v[i], (signs << (31 - (s * kAS + i))) & 0x80000000u);
             }
-            if (xlast == cur) {
+            const uint32_t m = (heads >> (s * kAS)) & ((1u << kAS) - 1u);
+            if (m == 0u) {
                 const float a = (v[0] + v[1]) + (v[2] + v[3]);
                 const float b = (v[4] + v[5]) + (v[6] + v[7]);
                 kahan_add(sum, comp, a + b);
             } else {
-                uint32_t xs[kAS];
-#pragma unroll
-                for (int i = 0; i < kAS; ++i) xs[i] = ex[2 * i];
 #pragma unroll
                 for (int i = 0; i < kAS; ++i) {
-                    if (xs[i] == kBad) break;
-                    if (xs[i] != cur) {
-                        flush(cur);
-                        cur = xs[i];
-                        ++nstart;
+                    if (m & (1u << i)) {
+                        flush();
+                        cur = __shfl_sync(0xffffffffu, x0, s * kAS + i);
                     }
                     kahan_add(sum, comp, v[i]);
                 }
             }
-            __syncwarp();
         }
-        flush(cur);
-        if (SINK != kSinkF64) finalize(32);
-        cp_async_wait<0>();
-        __syncwarp();
+        x0 = x1;
+        r0 = r1;
+        x1 = (uint32_t)(e2 >> 32);
+        r1 = (uint32_t)e2;
     }
+    flush();
+    if (SINK != kSinkF64) finalize(32);
+    cp_async_wait<0>();
     // (the local layout's runs are per segment: no distinct-bucket count)
-    if (count_runs && lane == 0 && nstart && !local) atomicAdd(stats + 1, (unsigned long long)nstart);
+    if (!LOCAL && count_runs && lane == 0 && nstart)
+        atomicAdd(stats + 1, (unsigned long long)nstart);
 }
 
 // The boundary elements of the window reduce.  Between task j - 1 and task j
@@ -1292,21 +1305,21 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
 // order (j first) in fp64, and stores the sum into ws.gexp.
 __global__ void __launch_bounds__(kThreads)
 k_window_combine(const unsigned long long* __restrict__ sorted_e,
-                 const unsigned long long* __restrict__ stats, int64_t npairs, int64_t G,
-                 WindowSink ws) {
+                 const unsigned long long* __restrict__ stats, int64_t npairs, int64_t per,
+                 int64_t G, WindowSink ws) {
     pdl_prologue();
     const int64_t total = (int64_t)(stats[0] < (unsigned long long)npairs ? stats[0] : npairs);
-    const int64_t ntasks = (total + kAPiece - 1) / kAPiece;
+    const int64_t ntasks = (total + per - 1) / per;
     const int lane = threadIdx.x & 31;
     auto xat = [&](int64_t i) { return (int64_t)(uint32_t)(__ldg(sorted_e + i) >> 32) * G; };
     auto xlast = [&](int64_t k) {
-        return xat(((k + 1) * kAPiece < total ? (k + 1) * kAPiece : total) - 1);
+        return xat(((k + 1) * per < total ? (k + 1) * per : total) - 1);
     };
     for (int64_t j = 1 + (int64_t)blockIdx.x * kWarps + (threadIdx.x >> 5); j < ntasks;
          j += (int64_t)gridDim.x * kWarps) {
-        const int64_t xfj = xat(j * kAPiece);
-        const int64_t xlp = xat(j * kAPiece - 1);
-        const int64_t xfn = (j + 1 < ntasks) ? xat((j + 1) * kAPiece) : INT64_MAX;
+        const int64_t xfj = xat(j * per);
+        const int64_t xlp = xat(j * per - 1);
+        const int64_t xfn = (j + 1 < ntasks) ? xat((j + 1) * per) : INT64_MAX;
         const int64_t e = xfj + lane;
         // shared with task j - 1, and no later boundary owns it
         bool open = e < xlp + 32 && e < xfn;
@@ -1315,7 +1328,7 @@ k_window_combine(const unsigned long long* __restrict__ sorted_e,
         for (int64_t kb = j; kb >= 0 && __any_sync(0xffffffffu, open); kb -= 32) {
             // lane i: bounds of task kb - i
             const int64_t kl = kb - lane;
-            const int64_t xfk = (kl >= 0) ? xat(kl * kAPiece) : INT64_MAX;
+            const int64_t xfk = (kl >= 0) ? xat(kl * per) : INT64_MAX;
             const int64_t xlk = (kl >= 0) ? xlast(kl) : 0;
             // tasks kb, kb - 1, ... holding e: the first ncnt of this round
             int ncnt = 0;
@@ -1519,22 +1532,63 @@ bool window_reduce_ok(const DevParams& p, const float* gout) {
     return p.Z == 32 && p.d % 32 == 0 && (((uintptr_t)gout & 15u) == 0);
 }
 
-int64_t window_records(int64_t npairs) { return (npairs + kAPiece - 1) / kAPiece; }
+// CTAs of the staged reduce per SM (at most 4 are resident; more give the
+// hardware ranges to balance with).  Measured on GB300, us per reduce:
+//                                   2      3      4      8     12
+//   global sort, rows read once   164    183    192    187    180   (Criteo-TB)
+//   global sort, rows re-read     245    200    195    190    190   (multi-hot)
+//   local sort                   43.1   44.4   44.0   41.7   42.2   (micro-benchmark)
+//                                99.9   99.1   96.6   90.8   89.0   (M = 2^26, batch 16384)
+//   window (deterministic)       95.6   79.7   77.9   77.7          (batch 20011), and its
+//   combine                       4.9    6.2    6.7   11.4
+// Rows read once in bucket order are random 128-byte HBM reads, of which fewer
+// in flight are served faster; the others wait for L2 and the reductions.
+constexpr int kWindowCtas = 3;
+static int staged_ctas(int sink, bool local, bool reread) {
+    if (sink == kSinkOnce) return kWindowCtas;
+    return local || reread ? 8 : 2;
+}
+
+// Entries per warp of the staged reduce over `entries` sorted entries.
+static int64_t staged_per(int64_t entries, int ctas, int sm_count) {
+    const int64_t warps = (int64_t)ctas * sm_count * kWarps;
+    const int64_t per = ((entries + warps - 1) / warps + 31) / 32 * 32;
+    return per < kAMinPer ? kAMinPer : per;
+}
+
+// At least the ranges of the window reduce of any batch of up to npairs pairs.
+int64_t window_records(int64_t npairs, int sm_count) {
+    const int64_t warps = (int64_t)kWindowCtas * sm_count * kWarps;
+    const int64_t most = (npairs + kAMinPer - 1) / kAMinPer;
+    return most < warps ? most : warps;
+}
+
+// The staged reduce over `entries` sorted entries, one range per warp.
+template <int SINK, bool LOCAL>
+static cudaError_t staged_reduce(const SortedBuffers& sb, int64_t npairs, int64_t entries,
+                                 const float* gout, bool reread, const DevParams& p, double* g,
+                                 const WindowSink& ws, const uint32_t* segn, bool count_runs,
+                                 int sm_count, cudaStream_t st) {
+    const int64_t per = staged_per(entries, staged_ctas(SINK, LOCAL, reread), sm_count);
+    const int64_t tasks = (entries + per - 1) / per;
+    const int grid = (int)((tasks + kWarps - 1) / kWarps);
+    auto kern = p.smask ? k_async_reduce<SINK, LOCAL, true> : k_async_reduce<SINK, LOCAL, false>;
+    return launch_k(kern, dim3(grid), dim3(kThreads), 0, st, sb.sorted_e, sb.stats, npairs, per,
+                    gout, reread, (uint32_t)p.G, g, ws, segn, count_runs);
+}
 
 cudaError_t launch_window_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
-                                 const DevParams& p, const WindowSink& ws, int sm_count,
-                                 cudaStream_t st) {
+                                 const DevParams& p, const WindowSink& ws, bool reread,
+                                 int sm_count, cudaStream_t st) {
     if (!window_reduce_ok(p, gout)) return cudaErrorInvalidValue;
-    const int64_t ntasks = window_records(npairs);   // upper bound
-    const int64_t blocks = (ntasks + kWarps - 1) / kWarps;
-    int grid = grid_for(k_async_reduce<kSinkOnce>, sm_count, blocks);
-    cudaError_t e = launch_k(k_async_reduce<kSinkOnce>, dim3(grid), dim3(kThreads), 0, st,
-                             sb.sorted_e, sb.stats, npairs, gout, p.G, p.smask,
-                             (double*)nullptr, ws, (const uint32_t*)nullptr, true);
+    const cudaError_t e = staged_reduce<kSinkOnce, false>(sb, npairs, npairs, gout, reread, p,
+                                                          nullptr, ws, nullptr, true, sm_count, st);
     if (e != cudaSuccess) return e;
-    grid = grid_for(k_window_combine, sm_count, blocks);
+    const int64_t per = staged_per(npairs, kWindowCtas, sm_count);
+    const int64_t ntasks = (npairs + per - 1) / per;   // upper bound
+    const int grid = grid_for(k_window_combine, sm_count, (ntasks + kWarps - 1) / kWarps);
     return launch_k(k_window_combine, dim3(grid), dim3(kThreads), 0, st, sb.sorted_e,
-                    (const unsigned long long*)sb.stats, npairs, p.G, ws);
+                    (const unsigned long long*)sb.stats, npairs, per, p.G, ws);
 }
 
 int64_t local_segments(int64_t npairs) { return (npairs + kLS - 1) / kLS; }
@@ -1562,19 +1616,16 @@ cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, ui
 
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
-                                 int sm_count, cudaStream_t st) {
+                                 bool reread, int sm_count, cudaStream_t st) {
     if (local && !window_reduce_ok(p, gout)) return cudaErrorInvalidValue;
     // 32-element chunks tiling the rows: asynchronous shared-memory staging
     if (window_reduce_ok(p, gout)) {
-        // 3 CTAs per SM (measured at the Criteo-TB shape: 0.170 ms against
-        // 0.177 with 4, the occupancy limit, 0.199 with 2 and 0.197 with 6):
-        // fewer random gathers in flight keep the DRAM more efficient
-        const int64_t ntasks = (npairs + kAPiece - 1) / kAPiece;   // upper bound
-        int grid = grid_for(k_async_reduce<kSinkF64>, sm_count, (ntasks + kWarps - 1) / kWarps);
-        if (grid > 3 * sm_count) grid = 3 * sm_count;
-        return launch_k(k_async_reduce<kSinkF64>, dim3(grid), dim3(kThreads), 0, st, sb.sorted_e,
-                        sb.stats, npairs, gout, p.G, p.smask, g, WindowSink{},
-                        local ? (const uint32_t*)sb.segn : (const uint32_t*)nullptr, count_runs);
+        if (local)
+            return staged_reduce<kSinkF64, true>(sb, npairs, local_segments(npairs) * kLS, gout,
+                                                 reread, p, g, WindowSink{}, sb.segn, false,
+                                                 sm_count, st);
+        return staged_reduce<kSinkF64, false>(sb, npairs, npairs, gout, reread, p, g, WindowSink{},
+                                              nullptr, count_runs, sm_count, st);
     }
     // blocks of 32+ elements: one warp per task, one element per lane
     if (p.L >= 32) {
