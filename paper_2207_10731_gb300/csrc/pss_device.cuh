@@ -140,6 +140,8 @@ struct Cols {
     int z[KC];     // offset of the column inside its chunk
     bool v[KC];    // column exists (d not a multiple of the group width)
     int e[KC];     // element offset of the column in the row
+    int js[KC];    // j and z, or 0 for a column that does not exist: a load
+    int zs[KC];    // through them is in range, and its value is not stored
     __device__ __forceinline__ Cols(const DevParams& p, int lg, int gs) {
         const int V = p.d / VW;
 #pragma unroll
@@ -149,6 +151,8 @@ struct Cols {
             e[k] = c * VW;
             j[k] = e[k] / p.Z;
             z[k] = e[k] - j[k] * p.Z;
+            js[k] = v[k] ? j[k] : 0;
+            zs[k] = v[k] ? z[k] : 0;
         }
     }
 };

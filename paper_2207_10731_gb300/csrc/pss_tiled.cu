@@ -17,6 +17,7 @@
 // 16-byte fp32 vector reductions, or one fp64 reduction per element with
 // consecutive lanes on consecutive elements (8 sectors per instruction).
 #include <climits>
+#include <type_traits>
 
 #include "pss_device.cuh"
 #include "pss_internal.h"
@@ -29,9 +30,8 @@ constexpr int kU = 4;            // ids in flight per group
 // at the multi-hot shape: 8 took 0.398 ms per forward with spills and 0.381
 // at 3 CTAs per SM, against 0.334 ms with 4)
 constexpr int kUM = 4;
-static_assert(kUM == 4 || kUM == 8, "the multi-id forward sums 4 or 8 values per round as a tree");
+static_assert(kUM == 4, "the multi-id forward sums 4 values per round as a tree");
 constexpr int kBagsPerGroup = 16;
-constexpr int kUB = 4;           // bags in flight per group in the forward's one-id path
 
 template <typename XT>
 struct Invalid;
@@ -104,17 +104,17 @@ __device__ __forceinline__ void stage_buckets(const DevParams& p, const int64_t*
     }
 }
 
-// One VW-wide load of a staged block (bucket x, column offset z); with signed
-// hashing (SG) the bucket carries the sign in bit 31, applied to the value.
-// G < 2^31 (an int32 of the API): with 32-bit buckets the element index is
-// one 32 x 32 -> 64-bit multiply.
+// One VW-wide load of the block of a staged bucket x; wz points at the column
+// in the array's first block, Gb is the bytes between block starts (below 2^32
+// with 32-bit buckets: one multiply-add).  With signed hashing (SG) the bucket
+// carries the sign in bit 31, applied to the value.
 template <bool SG, typename V, typename XT>
-__device__ __forceinline__ typename V::T gather(const float* __restrict__ w, uint64_t G, XT x, int z) {
+__device__ __forceinline__ typename V::T gather(const float* __restrict__ wz, uint64_t Gb, XT x) {
     const XT xb = SG ? (x & ~(XT)0x80000000u) : x;
-    const uint64_t e = (sizeof(XT) == 4) ? (uint64_t)(uint32_t)G * (uint32_t)xb + (uint32_t)z
-                                         : G * (uint64_t)xb + (uint64_t)z;
-    if (!SG) return V::ldg(w + e);
-    return sign_by(V::ldg(w + e), (uint32_t)x & 0x80000000u);
+    const uint64_t off = (sizeof(XT) == 4) ? (uint64_t)(uint32_t)Gb * (uint32_t)xb
+                                           : Gb * (uint64_t)xb;
+    const auto v = V::ldg(reinterpret_cast<const float*>(reinterpret_cast<const char*>(wz) + off));
+    return SG ? sign_by(v, (uint32_t)x & 0x80000000u) : v;
 }
 
 // ---------------------------------------------------------------------------
@@ -123,256 +123,510 @@ __device__ __forceinline__ typename V::T gather(const float* __restrict__ w, uin
 // other (no CTA-wide barrier): the lanes hash the tile's (id, chunk) pairs
 // 32 at a time, then the lane groups gather and sum-pool their bags.
 constexpr int kWarpPairs = 512;   // staged pairs per warp and round
+constexpr int kMaxTileBags = 32;  // bags per tile at most: one lane each
+constexpr int kIdU = 4;           // ids in flight per lane while a window is hashed
 
-// Hash the pairs [0, nq*J) of ids qc0.. into s_x (warp-cooperative); emits
-// the buckets for the sorted backward when asked.
+
+// Variants of the forward (MODE): rows in flight per lane group in one-id
+// tiles, and CTAs per SM.  Measured on GB300, us per forward with the kernel
+// compiled for 3, 2 and 4 CTAs per SM (and 4, 16 and 4 rows in flight):
+//                                 3      2      4
+//   Criteo-TB shape, B = 65536  154    152    199
+//   M = 2^26, B = 16384          63     57     99
+//   Criteo-TB shape, B = 2048   9.4   10.0   10.3
+//   multi-hot, 20 ids per bag   261    288    247
+//   multi-hot, 5 ids per bag    148    ---    138
+// HBM takes the rows of few warps that write many at a time best; long bags
+// want warps.
+constexpr int kFwdShort = 0;   // one-id bags
+constexpr int kFwdMany = 1;    // many one-id bags, rows of a whole warp
+constexpr int kFwdLong = 2;    // bags of several ids
+constexpr int fwd_rows(int mode) { return mode == kFwdMany ? 16 : 4; }
+constexpr int fwd_min_ctas(int VW, int KC, int mode) {
+    return KC * VW > 4 ? (KC * VW <= 8 ? 2 : 1)
+                       : mode == kFwdMany ? 2 : mode == kFwdLong && KC == 1 ? 4 : 3;
+}
+
+// Bucket of a pair from its hash s = (A*key + B0) mod P: s mod R, the same
+// integers as hash_bucket.  For R <= 2^30, q is floor(s / R) or up to 3 less:
+// Barrett's quotient loses 1 (see hash_bucket) and the three dropped parts of
+// the 64 x 64-bit product lose less than 1 each; so s - q*R < 4R <= 2^32 and
+// 32-bit arithmetic modulo 2^32 gives it.
+template <typename XT>
+__device__ __forceinline__ XT mod_R(const DevParams& p, uint64_t s) {
+    if (sizeof(XT) == 4 && p.R <= (uint64_t(1) << 30)) {
+        const uint32_t sh = (uint32_t)(s >> 32), sl = (uint32_t)s;
+        const uint32_t rh = (uint32_t)(p.Rinv >> 32), rl = (uint32_t)p.Rinv;
+        const uint32_t R = (uint32_t)p.R;
+        const uint32_t q = sh * rh + __umulhi(sh, rl) + __umulhi(sl, rh);
+        uint32_t r = sl - q * R;
+        r = min(r, r - 2u * R);   // (wraps above r when r is the smaller)
+        return (XT)min(r, r - R);
+    }
+    const uint64_t q = __umul64hi(s, p.Rinv);
+    const uint64_t R = sizeof(XT) == 4 ? (uint64_t)(uint32_t)p.R : p.R;
+    const uint64_t r = s - q * R;
+    return (XT)(r >= R ? r - R : r);
+}
+
+// a + b mod P for a, b < P
+__device__ __forceinline__ uint64_t add_p61(uint64_t a, uint64_t b) {
+    const uint64_t s = a + b;
+    return s >= kP61 ? s - kP61 : s;
+}
+
+// Two fp32 operations per instruction (each rounded as the scalar one).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {   // a - b = fma(b, -1, a)
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+    return r;
+}
+
+// Compensated sums of VW-wide columns: add(v) is kahan_add per element,
+// add4 the tree sum of four values first; merge adds another lane's sum (the
+// compensations are added plainly: their rounding is of second order).
+template <int VW>
+struct Sum;
+template <>
+struct Sum<4> {
+    uint64_t s0 = 0, s1 = 0, c0 = 0, c1 = 0;
+    static __device__ __forceinline__ void kahan(uint64_t& s, uint64_t& c, uint64_t x) {
+        const uint64_t y = sub2(x, c);
+        const uint64_t t = add2(s, y);
+        c = sub2(sub2(t, s), y);
+        s = t;
+    }
+    __device__ __forceinline__ void add4(const float4& a, const float4& b, const float4& c,
+                                         const float4& d) {
+        kahan(s0, c0, add2(add2(pack2(a.x, a.y), pack2(b.x, b.y)),
+                           add2(pack2(c.x, c.y), pack2(d.x, d.y))));
+        kahan(s1, c1, add2(add2(pack2(a.z, a.w), pack2(b.z, b.w)),
+                           add2(pack2(c.z, c.w), pack2(d.z, d.w))));
+    }
+    __device__ __forceinline__ void merge(int o) {
+        const uint64_t t0 = __shfl_xor_sync(0xffffffffu, s0, o);
+        const uint64_t t1 = __shfl_xor_sync(0xffffffffu, s1, o);
+        const uint64_t d0 = __shfl_xor_sync(0xffffffffu, c0, o);
+        const uint64_t d1 = __shfl_xor_sync(0xffffffffu, c1, o);
+        kahan(s0, c0, t0);
+        kahan(s1, c1, t1);
+        c0 = add2(c0, d0);
+        c1 = add2(c1, d1);
+    }
+    __device__ __forceinline__ float4 value() const {
+        float4 v;
+        unpack2(sub2(s0, c0), v.x, v.y);
+        unpack2(sub2(s1, c1), v.z, v.w);
+        return v;
+    }
+};
+template <>
+struct Sum<1> {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add4(float a, float b, float x, float y) {
+        kahan_add(s, c, (a + b) + (x + y));
+    }
+    __device__ __forceinline__ void merge(int o) {
+        const float os = __shfl_xor_sync(0xffffffffu, s, o);
+        const float oc = __shfl_xor_sync(0xffffffffu, c, o);
+        kahan_add(s, c, os);
+        c += oc;
+    }
+    __device__ __forceinline__ float value() const { return s - c; }
+};
+
+// How a forward's work is cut.  One-id bags: tiles of wb consecutive bags of
+// one table; 2^log2pw >= wb lanes own one bag each (32 >> log2pw lanes per
+// bag).  Longer bags: 2^log2pi ids are hashed at a time, 32 >> log2pi lanes
+// each.  stepA[k] and stepA2[k] are A and A2 times the lanes per bag (k = 0)
+// or id (1), mod P.
+struct FwdGeom {
+    int wb, log2pw, log2pi, tiles_per_table;
+    uint64_t stepA[2], stepA2[2];
+    uint64_t TJ;          // T * J: keys of consecutive ids
+    uint64_t Gb;          // bytes between block starts
+};
+
+// Buckets of chunks j0, j0 + lpi, ... of one id into sx[0 .. J), Invalid for a
+// bad id: one product A*key per lane, chunk j + lpi has step = A*lpi more.
 template <typename XT, bool SG>
-__device__ __forceinline__ void warp_stage(const DevParams& p, const int64_t* __restrict__ idx,
-                                           int t, uint64_t card, int64_t qc0, int nq, XT* s_x,
-                                           DevError* err, uint32_t* __restrict__ pair_x,
+__device__ __forceinline__ void hash_id(const DevParams& p, uint64_t TJ, uint64_t id, uint32_t tJ,
+                                        bool valid, int j0, int lpi, uint64_t step, uint64_t step2,
+                                        XT* sx) {
+    const uint64_t key = id * TJ + tJ + (uint32_t)j0;   // hash_key; tJ = t*J
+    uint64_t s = affine_mod_p61(p.A, key, p.B0);
+    uint64_t s2 = SG ? affine_mod_p61(p.A2, key, p.B2) : 0ull;
+    for (int j = j0; j < p.J; j += lpi) {
+        XT x = mod_R<XT>(p, s);
+        s = add_p61(s, step);
+        if (SG) {
+            x |= (XT)((uint32_t)(s2 & 1u) << 31);
+            s2 = add_p61(s2, step2);
+        }
+        sx[j] = valid ? x : Invalid<XT>::v;
+    }
+}
+
+// n staged buckets to pair_x + at, whose ids are consecutive.
+template <typename XT>
+__device__ __forceinline__ void emit_pairs(const XT* s_x, int n, int J, uint32_t* __restrict__ px,
                                            int lane) {
-    const int npairs = nq * p.J;
-    const bool jpow2 = (p.J & (p.J - 1)) == 0;
-    const int log2J = 31 - __clz(p.J);
-    for (int base = 0; base < npairs; base += 32) {
-        const int k = base + lane;
-        XT x = Invalid<XT>::v;
-        if (k < npairs) {
-            const int qi = jpow2 ? (k >> log2J) : k / p.J;
-            const int j = k - qi * p.J;
-            const int64_t q = qc0 + qi;
-            const int64_t id = __ldg(idx + q);
-            if ((uint64_t)id < card) {
-                const uint64_t key = hash_key(p, (uint64_t)id, t, j);
-                x = (XT)hash_bucket(p, key);
-                if (SG) x |= (XT)hash_sign_bit(p, key);
-            } else if (j == 0) {
-                record_bad_id(err, q);
-            }
-            s_x[k] = x;
-            if (pair_x) pair_x[qc0 * p.J + k] = (uint32_t)x;
-        }
+    if (sizeof(XT) == 4 && (J & 3) == 0) {
+        for (int k = lane; k < n / 4; k += 32)
+            reinterpret_cast<uint4*>(px)[k] = reinterpret_cast<const uint4*>(s_x)[k];
+    } else if (sizeof(XT) == 4 && (J & 1) == 0) {
+        for (int k = lane; k < n / 2; k += 32)
+            reinterpret_cast<uint2*>(px)[k] = reinterpret_cast<const uint2*>(s_x)[k];
+    } else {
+        for (int k = lane; k < n; k += 32) px[k] = (uint32_t)s_x[k];
     }
-    __syncwarp();
 }
 
-// One-id tiles: stage by BAG.  s_x[bb*J + j] is the bucket of chunk j of the
-// id of bag bb (Invalid for an empty bag or a bad id), so the gather needs no
-// offsets; the id's output row is written here too.
-template <typename XT, bool SG>
-__device__ __forceinline__ void warp_stage_bags(const DevParams& p, const int64_t* __restrict__ idx,
-                                                int t, uint64_t card, const int64_t* s_off, int nb,
-                                                XT* s_x, DevError* err,
-                                                uint32_t* __restrict__ pair_x,
-                                                uint32_t* __restrict__ q_row, uint32_t row0,
-                                                int lane) {
-    const int npairs = nb * p.J;
-    const bool jpow2 = (p.J & (p.J - 1)) == 0;
-    const int log2J = 31 - __clz(p.J);
-    for (int base = 0; base < npairs; base += 32) {
-        const int k = base + lane;
-        XT x = Invalid<XT>::v;
-        if (k < npairs) {
-            const int bb = jpow2 ? (k >> log2J) : k / p.J;
-            const int j = k - bb * p.J;
-            const int64_t q = s_off[bb];
-            if (s_off[bb + 1] > q) {
-                const int64_t id = __ldg(idx + q);
-                if ((uint64_t)id < card) {
-                    const uint64_t key = hash_key(p, (uint64_t)id, t, j);
-                    x = (XT)hash_bucket(p, key);
-                if (SG) x |= (XT)hash_sign_bit(p, key);
-                } else if (j == 0) {
-                    record_bad_id(err, q);
-                }
-                if (pair_x) pair_x[q * p.J + j] = (uint32_t)x;
-                if (q_row && j == 0) q_row[q] = row0 + (uint32_t)bb * (uint32_t)p.T;
-            }
-            s_x[k] = x;
-        }
-    }
-    __syncwarp();
-}
-
+// Bags of any length: pools the nb bags of a tile, lane l holding the offsets
+// [q0, q1) of bag l (mod the power of two at or above the tile's bags), all
+// ids within [qa, qb).  The ids are staged and hashed in windows; the whole
+// warp takes one bag at a time; its ng lane groups add ng consecutive ids of
+// the bag in parallel, kUM steps per round.  A round's kUM values are summed
+// as a tree and added with compensation; at the end of the bag the groups'
+// sums are merged the same way and group 0 stores the row.
+// What bounds it: instruction issue, then the L2 gathers.  So whole rounds of
+// valid ids run without tests, the sums take two elements per instruction, an
+// id's chunks are hashed from one product, and a bag's bounds in the window
+// are 32-bit numbers that the lanes compute together.
 template <int VW, int KC, typename XT, bool SG>
-__global__ void __launch_bounds__(kThreads, (KC == 1) ? 4 : 1)
-k_forward_warp(DevParams p, const int64_t* __restrict__ idx, int64_t nnz,
+__device__ __forceinline__ void
+forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ idx, uint32_t tJ,
+             uint64_t card, int64_t q0, int64_t q1, int nb, XT* s_x,
+             const float* const (&wz)[KC], const Cols<VW, KC>& col, float* orow, int64_t ostride,
+             uint32_t row, DevError* err, uint32_t* __restrict__ pair_x,
+             uint32_t* __restrict__ q_row, int log2gs, int lane) {
+    using V = Vec<VW>;
+    using VT = typename V::T;
+    const int gs = 1 << log2gs;
+    const int g = lane >> log2gs;
+    const int ng = 32 >> log2gs;
+    const int J = p.J;
+    const int sJ = ng * J;                   // staged buckets from one of a lane's ids to the next
+    const int gJ = g * J;
+    const int qcw = kWarpPairs / J;          // ids per staged window
+    const int ids = 1 << fg.log2pi, lpi = 32 >> fg.log2pi;
+    const int64_t qb = __shfl_sync(0xffffffffu, q1, nb - 1);
+    int64_t sw0 = __shfl_sync(0xffffffffu, q0, 0);
+    int bi = 0;
+    Sum<VW> acc[KC];
+    for (;;) {
+        // stage the window [sw0, sw0 + n)
+        const int n = (int)((qb - sw0) < qcw ? (qb - sw0) : qcw);
+        bool ok = true;
+        for (int i0 = lane & (ids - 1); i0 < n; i0 += ids * kIdU) {
+            int64_t id[kIdU];   // loads in flight together
+#pragma unroll
+            for (int u = 0; u < kIdU; ++u)
+                id[u] = i0 + u * ids < n ? __ldg(idx + sw0 + i0 + u * ids) : 0;
+#pragma unroll
+            for (int u = 0; u < kIdU; ++u) {
+                const int i = i0 + u * ids;
+                if (i >= n) break;
+                const bool valid = (uint64_t)id[u] < card;
+                ok &= valid;
+                if (!valid && lane < ids) record_bad_id(err, sw0 + i);
+                hash_id<XT, SG>(p, fg.TJ, (uint64_t)id[u], tJ, valid, lane >> fg.log2pi, lpi,
+                                fg.stepA[1], fg.stepA2[1], s_x + i * J);
+            }
+        }
+        const bool clean = __all_sync(0xffffffffu, ok);   // every id valid
+        __syncwarp();
+        if (pair_x) emit_pairs<XT>(s_x, n * J, J, pair_x + sw0 * J, lane);
+        // this lane's bag inside the window, and whether it ends there
+        const int64_t a = q0 - sw0, c = q1 - sw0;
+        const int lo = (int)(a < 0 ? 0 : a < n ? a : n), hi = (int)(c < n ? c : n);
+        const unsigned ends = __ballot_sync(0xffffffffu, c <= n);
+        for (; bi < nb; ++bi) {
+            const int b0 = __shfl_sync(0xffffffffu, lo, bi), b1 = __shfl_sync(0xffffffffu, hi, bi);
+            if (q_row)   // the bag's ids' output row, one store per lane
+                for (int i = b0 + lane; i < b1; i += 32) q_row[sw0 + i] = row;
+            const XT* sx = s_x + b0 * J;
+            int left = b1 - b0;   // ids to add
+            if (clean) {
+                // whole rounds: every group has kUM ids
+                for (; left >= kUM * ng; left -= kUM * ng) {
+                    VT v[kUM][KC];
+#pragma unroll
+                    for (int u = 0; u < kUM; ++u)
+#pragma unroll
+                        for (int k = 0; k < KC; ++k)
+                            v[u][k] = gather<SG, V>(wz[k], fg.Gb, sx[gJ + u * sJ + col.js[k]]);
+                    sx += kUM * sJ;
+#pragma unroll
+                    for (int k = 0; k < KC; ++k) acc[k].add4(v[0][k], v[1][k], v[2][k], v[3][k]);
+                }
+                // the rest: lanes past the bag load its next id and drop it
+                if (left > 0) {
+                    VT v[kUM][KC];
+#pragma unroll
+                    for (int u = 0; u < kUM; ++u) {
+                        const bool in = g + u * ng < left;
+                        const int o = in ? gJ + u * sJ : 0;
+#pragma unroll
+                        for (int k = 0; k < KC; ++k) {
+                            v[u][k] = gather<SG, V>(wz[k], fg.Gb, sx[o + col.js[k]]);
+#pragma unroll
+                            for (int i = 0; i < VW; ++i)
+                                V::set(v[u][k], i, in ? V::get(v[u][k], i) : 0.f);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < KC; ++k) acc[k].add4(v[0][k], v[1][k], v[2][k], v[3][k]);
+                }
+            } else {
+                for (int i0 = g; i0 - g < left; i0 += kUM * ng) {
+                    VT v[kUM][KC];
+#pragma unroll
+                    for (int u = 0; u < kUM; ++u)
+#pragma unroll
+                        for (int k = 0; k < KC; ++k) {
+#pragma unroll
+                            for (int i = 0; i < VW; ++i) V::set(v[u][k], i, 0.f);
+                            if (i0 + u * ng < left) {
+                                const XT x = sx[(i0 + u * ng) * J + col.js[k]];
+                                if (x != Invalid<XT>::v) v[u][k] = gather<SG, V>(wz[k], fg.Gb, x);
+                            }
+                        }
+#pragma unroll
+                    for (int k = 0; k < KC; ++k) acc[k].add4(v[0][k], v[1][k], v[2][k], v[3][k]);
+                }
+            }
+            if (!((ends >> bi) & 1u)) break;   // it goes on in the next window
+            for (int o = gs; o < 32; o <<= 1)
+#pragma unroll
+                for (int k = 0; k < KC; ++k) acc[k].merge(o);
+            if (g == 0) {
+#pragma unroll
+                for (int k = 0; k < KC; ++k)
+                    if (col.v[k]) V::stcs(orow + col.e[k], acc[k].value());
+            }
+            orow += ostride;
+            row += (uint32_t)p.T;
+#pragma unroll
+            for (int k = 0; k < KC; ++k) acc[k] = Sum<VW>();
+        }
+        if (bi >= nb) break;
+        sw0 += n;
+        __syncwarp();   // s_x is staged again
+    }
+}
+
+// What bounds it with one-id bags: the pooled rows' stores to HBM at d = 128
+// (one 16-byte load and store per lane and row), and the latency of the chain
+// offsets -> ids -> hash -> blocks behind them.  So a warp loads the offsets
+// of the tile after next and the ids of the next tile before it gathers its
+// own, and in tiles whose bags all hold one valid id a row costs one
+// shared-memory load, one multiply-add, one load and one store.  Tiles run
+// over the tables of a range of bags first, so that the rows that the GPU
+// writes at a time are one contiguous piece of the output.
+template <int VW, int KC, typename XT, bool SG, int MODE>
+__global__ void __launch_bounds__(kThreads, fwd_min_ctas(VW, KC, MODE))
+k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ idx, int64_t nnz,
                const int64_t* __restrict__ off, int64_t B, const float* __restrict__ w,
                float* __restrict__ out, DevError* err, uint32_t* __restrict__ pair_x,
-               uint32_t* __restrict__ q_row, int log2gs, int wb,
-               int tiles_per_table, int64_t b_lo, int64_t b_hi) {
+               uint32_t* __restrict__ q_row, int log2gs, const __grid_constant__ FwdGeom fg,
+               int64_t b_lo, int64_t b_hi) {
     pdl_prologue();
     using V = Vec<VW>;
     using VT = typename V::T;
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    int64_t* s_off = reinterpret_cast<int64_t*>(smem) + warp * (wb + 1);
-    XT* s_x = reinterpret_cast<XT*>(reinterpret_cast<int64_t*>(smem) + kWarps * (wb + 1)) +
-              warp * kWarpPairs;
+    XT* s_x = reinterpret_cast<XT*>(smem) + warp * kWarpPairs;
     const int gs = 1 << log2gs;
     const int lg = lane & (gs - 1);
     const int g = lane >> log2gs;
+    const int wb = fg.wb;
     const int bpg = wb >> (5 - log2gs);      // bags per group
     const Cols<VW, KC> col(p, lg, gs);
-    const uint64_t G = (uint64_t)p.G;
+    const float* wz[KC];
+#pragma unroll
+    for (int k = 0; k < KC; ++k) wz[k] = w + col.zs[k];
     const int J = p.J;
-    const int qcw = kWarpPairs / J;          // ids per staging round
-    const int64_t ntiles = (int64_t)p.T * tiles_per_table;
     const int64_t ostride = (int64_t)p.T * p.d;
+    const int tpt = fg.tiles_per_table;
+    const int bag = lane & ((1 << fg.log2pw) - 1);   // this lane's bag of the tile
+    const int j0 = lane >> fg.log2pw;                // its first chunk
+    const int lpb = 32 >> fg.log2pw;                 // lanes per bag
 
-    for (int64_t tile = (int64_t)blockIdx.x * kWarps + warp; tile < ntiles;
-         tile += (int64_t)gridDim.x * kWarps) {
-        // ntiles < 2^31 (checked by the launcher): 32-bit division
-        const int t = (int)((uint32_t)tile / (uint32_t)tiles_per_table);
-        const int64_t b0 = b_lo + (tile - (int64_t)t * tiles_per_table) * wb;
+    // tiles of this warp: tile number = r * T + t (below 2^30, checked by the
+    // launcher), advanced without divisions, and with it the place of the
+    // lane's bag in the offsets
+    const int nwarps = (int)gridDim.x * kWarps;
+    const int step_r = nwarps / p.T, step_t = nwarps - step_r * p.T;
+    const int64_t step_o = (int64_t)step_t * B + (int64_t)step_r * wb;
+    const int64_t wrap_o = wb - (int64_t)p.T * B;
+    int r = ((int)blockIdx.x * kWarps + warp) / p.T;
+    int t = ((int)blockIdx.x * kWarps + warp) - r * p.T;
+    if (r >= tpt) return;
+    const int64_t* po = off + (int64_t)t * B + b_lo + (int64_t)r * wb + bag;
+    const int64_t nbags = b_hi - b_lo;
+    auto advance = [&](int& tt, int& rr) {
+        tt += step_t;
+        rr += step_r;
+        po += step_o;
+        if (tt >= p.T) {
+            tt -= p.T;
+            ++rr;
+            po += wrap_o;
+        }
+    };
+    // offsets of this lane's bag of tile row rr at po: a zero-length bag past the end
+    auto load_offsets = [&](int rr, int64_t& q0, int64_t& q1) {
+        q0 = q1 = 0;
+        if (bag < wb && (int64_t)rr * wb + bag < nbags) {
+            q0 = __ldg(po);
+            q1 = __ldg(po + 1);
+        }
+    };
+    // the id of a bag that holds exactly one (offsets in range), else -1
+    auto load_id = [&](int64_t q0, int64_t q1) -> int64_t {
+        return (q0 >= 0 && q1 == q0 + 1 && q1 <= nnz) ? __ldg(idx + q0) : -1;
+    };
+
+    int64_t q0, q1, q0n, q1n;
+    load_offsets(r, q0, q1);
+    int t1 = t, r1 = r;
+    advance(t1, r1);
+    load_offsets(r1, q0n, q1n);
+    int64_t id = load_id(q0, q1);
+    while (r < tpt) {
+        int t2 = t1, r2 = r1;
+        advance(t2, r2);
+        const int64_t idn = load_id(q0n, q1n);
+        int64_t q0m, q1m;
+        load_offsets(r2, q0m, q1m);
+
+        const int64_t b0 = b_lo + (int64_t)r * wb;
         const int nb = (int)((b_hi - b0) < wb ? (b_hi - b0) : wb);
-        const int64_t s0 = (int64_t)t * B + b0;
-        float* obase = out + ((b0 * p.T) + t) * (int64_t)p.d;
-        const int gb0 = min(g * bpg, nb);
-        const int gb1 = min(gb0 + bpg, nb);
-
-        for (int i = lane; i <= nb; i += 32) s_off[i] = __ldg(off + s0 + i);
-        __syncwarp();
-        bool bad = false, multi = false;
-        for (int i = lane; i < nb; i += 32) {
-            const int64_t a = s_off[i], c = s_off[i + 1];
-            bad |= (a < 0 || c < a || c > nnz);
-            multi |= (c - a > 1);
-        }
-        bad = __any_sync(0xffffffffu, bad);
-        multi = __any_sync(0xffffffffu, multi);
-        if (bad) {
-            if (lane == 0) record_bad_offsets(err);
-            for (int bi = gb0; bi < gb1; ++bi)
-#pragma unroll
-                for (int k = 0; k < KC; ++k) {
-                    if (!col.v[k]) continue;
-                    VT z;
-#pragma unroll
-                    for (int i = 0; i < VW; ++i) V::set(z, i, 0.f);
-                    V::stcs(obase + bi * ostride + col.e[k], z);
-                }
-            __syncwarp();
-            continue;
-        }
+        float* obase = out + b0 * ostride + (int64_t)t * p.d;
+        const uint32_t row0 = (uint32_t)b0 * (uint32_t)p.T + (uint32_t)t;
+        const uint32_t tJ = (uint32_t)t * (uint32_t)J;
         const uint64_t card = (uint64_t)__ldg(p.cards + t);
-        const int64_t qb = s_off[nb];
-
-        if (!multi && nb * J <= kWarpPairs) {
-            // every bag holds at most one id: one load per bag, no accumulation
-            warp_stage_bags<XT, SG>(p, idx, t, card, s_off, nb, s_x, err, pair_x, q_row,
-                                (uint32_t)(b0 * p.T + t), lane);
-            float* orow0 = obase + gb0 * ostride;
-            for (int bb0 = gb0; bb0 < gb1; bb0 += kUB) {
-                VT v[kUB][KC];
+        const bool has = q1 > q0;
+        const unsigned odd = __ballot_sync(0xffffffffu, q0 < 0 || q1 < q0 || q1 > nnz);
+        const bool multi = __any_sync(0xffffffffu, q1 - q0 > 1) || nb * J > kWarpPairs;
+        if (odd | (unsigned)multi) {
+            if (odd) {
+                if (lane == 0) record_bad_offsets(err);
+                for (int bi = g; bi < nb; bi += 32 >> log2gs)
 #pragma unroll
-                for (int u = 0; u < kUB; ++u) {
-                    const int bb = bb0 + u;
+                    for (int k = 0; k < KC; ++k) {
+                        if (!col.v[k]) continue;
+                        VT z;
+#pragma unroll
+                        for (int i = 0; i < VW; ++i) V::set(z, i, 0.f);
+                        V::stcs(obase + bi * ostride + col.e[k], z);
+                    }
+            } else {
+                forward_bags<VW, KC, XT, SG>(p, fg, idx, tJ, card, q0, q1, nb, s_x, wz, col, obase,
+                                             ostride, row0, err, pair_x, q_row, log2gs, lane);
+            }
+        } else {
+            // every bag holds at most one id: s_x[bag*J + j] is the bucket of
+            // chunk j of the bag's id (Invalid for an empty bag or a bad id),
+            // one load per bag, no accumulation
+            const bool mine = bag < nb;
+            const bool valid = has && (uint64_t)id < card;
+            if (mine)
+                hash_id<XT, SG>(p, fg.TJ, (uint64_t)id, tJ, valid, j0, lpb, fg.stepA[0],
+                                fg.stepA2[0], s_x + bag * J);
+            if (has && j0 == 0) {
+                if (!valid) record_bad_id(err, q0);
+                if (q_row) q_row[q0] = row0 + (uint32_t)bag * (uint32_t)p.T;
+            }
+            __syncwarp();
+            if (pair_x) {
+                // the bags' ids are consecutive; empty bags have no pair
+                if (__all_sync(0xffffffffu, has || !mine)) {
+                    emit_pairs<XT>(s_x, nb * J, J,
+                                   pair_x + __shfl_sync(0xffffffffu, q0, 0) * J, lane);
+                } else if (has) {
+                    for (int j = j0; j < J; j += lpb)
+                        pair_x[q0 * J + j] = (uint32_t)s_x[bag * J + j];
+                }
+            }
+            const int gb0 = min(g * bpg, nb);
+            float* orow = obase + gb0 * ostride;
+            const XT* sx = s_x + gb0 * J;
+            int n = min(bpg, nb - gb0);
+            if (nb == wb && __all_sync(0xffffffffu, valid || !mine)) {
+                // whole tile, all ids valid: no tests in the rows' loops
+                auto rows = [&](auto nu) {
+                    constexpr int U = decltype(nu)::value;
+                    VT v[U][KC];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+#pragma unroll
+                        for (int k = 0; k < KC; ++k)
+                            v[u][k] = gather<SG, V>(wz[k], fg.Gb, sx[col.js[k]]);
+                        sx += J;
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+#pragma unroll
+                        for (int k = 0; k < KC; ++k)
+                            if (col.v[k]) V::stcs(orow + col.e[k], v[u][k]);
+                        orow += ostride;
+                    }
+                    n -= U;
+                };
+                constexpr int kRows = fwd_rows(MODE);
+                if (kRows > 4)
+                    while (n >= kRows) rows(std::integral_constant<int, kRows>());
+                while (n >= 4) rows(std::integral_constant<int, 4>());
+            }
+            constexpr int kU4 = 4;
+            for (; __any_sync(0xffffffffu, n > 0); n -= kU4) {
+                VT v[kU4][KC];
+#pragma unroll
+                for (int u = 0; u < kU4; ++u)
 #pragma unroll
                     for (int k = 0; k < KC; ++k) {
 #pragma unroll
                         for (int i = 0; i < VW; ++i) V::set(v[u][k], i, 0.f);
-                        if (bb < gb1 && col.v[k]) {
-                            const XT x = s_x[bb * J + col.j[k]];
-                            if (x != Invalid<XT>::v) v[u][k] = gather<SG, V>(w, G, x, col.z[k]);
+                        if (u < n && col.v[k]) {
+                            const XT x = sx[u * J + col.j[k]];
+                            if (x != Invalid<XT>::v) v[u][k] = gather<SG, V>(wz[k], fg.Gb, x);
                         }
                     }
-                }
 #pragma unroll
-                for (int u = 0; u < kUB; ++u) {
-                    if (bb0 + u >= gb1) break;
+                for (int u = 0; u < kU4; ++u)
 #pragma unroll
                     for (int k = 0; k < KC; ++k)
-                        if (col.v[k]) V::stcs(orow0 + col.e[k], v[u][k]);
-                    orow0 += ostride;
-                }
-            }
-            __syncwarp();
-            continue;
-        }
-
-        // general bags: the whole warp takes one bag at a time; its ng lane
-        // groups add ng consecutive ids of the bag in parallel, kUM steps per
-        // round.  A round's kUM values are summed as a tree and added to the
-        // running sum with compensation (Kahan); at the end of the bag the
-        // groups' sums are merged the same way and group 0 stores the row.
-        const int ng = 32 >> log2gs;
-        int64_t sw0 = 0, sw1 = 0;        // ids staged in s_x: [sw0, sw1)
-        for (int bi = 0; bi < nb; ++bi) {
-            const int64_t a = s_off[bi], c = s_off[bi + 1];
-            float acc[KC][VW], cmp[KC][VW];
-#pragma unroll
-            for (int k = 0; k < KC; ++k)
-#pragma unroll
-                for (int i = 0; i < VW; ++i) acc[k][i] = cmp[k][i] = 0.f;
-            const uint32_t row = (uint32_t)((b0 + bi) * p.T + t);
-            for (int64_t q = a; q < c;) {
-                if (q >= sw1) {
-                    sw0 = q;
-                    sw1 = (qb - q) < qcw ? qb : q + qcw;
-                    warp_stage<XT, SG>(p, idx, t, card, sw0, (int)(sw1 - sw0), s_x, err, pair_x,
-                                       lane);
-                }
-                const int64_t qend = c < sw1 ? c : sw1;
-                // ids of the staged window by their 32-bit offset in it
-                const int i1 = (int)(qend - sw0);
-                for (int is = (int)(q - sw0); is < i1; is += kUM * ng) {
-                    VT v[kUM][KC];
-#pragma unroll
-                    for (int u = 0; u < kUM; ++u) {
-                        const int ii = is + u * ng + g;
-#pragma unroll
-                        for (int k = 0; k < KC; ++k) {
-#pragma unroll
-                            for (int i = 0; i < VW; ++i) V::set(v[u][k], i, 0.f);
-                            if (ii < i1 && col.v[k]) {
-                                const XT x = s_x[ii * J + col.j[k]];
-                                if (x != Invalid<XT>::v) v[u][k] = gather<SG, V>(w, G, x, col.z[k]);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int k = 0; k < KC; ++k)
-#pragma unroll
-                        for (int i = 0; i < VW; ++i) {
-                            float r = (V::get(v[0][k], i) + V::get(v[1][k], i)) +
-                                      (V::get(v[2][k], i) + V::get(v[3][k], i));
-                            if (kUM == 8)
-                                r += (V::get(v[kUM / 2][k], i) + V::get(v[kUM / 2 + 1][k], i)) +
-                                     (V::get(v[kUM - 2][k], i) + V::get(v[kUM - 1][k], i));
-                            kahan_add(acc[k][i], cmp[k][i], r);
-                        }
-                }
-                q = qend;
-            }
-            // the bag's ids' output row, one store per lane
-            if (q_row)
-                for (int64_t qq = a + lane; qq < c; qq += 32) q_row[qq] = row;
-            for (int o = gs; o < 32; o <<= 1) {
-#pragma unroll
-                for (int k = 0; k < KC; ++k)
-#pragma unroll
-                    for (int i = 0; i < VW; ++i) {
-                        const float os = __shfl_xor_sync(0xffffffffu, acc[k][i], o);
-                        const float oc = __shfl_xor_sync(0xffffffffu, cmp[k][i], o);
-                        kahan_add(acc[k][i], cmp[k][i], os);
-                        kahan_add(acc[k][i], cmp[k][i], -oc);
-                    }
-            }
-            if (g == 0) {
-                float* orow = obase + bi * ostride;
-#pragma unroll
-                for (int k = 0; k < KC; ++k) {
-                    if (!col.v[k]) continue;
-                    VT o;
-#pragma unroll
-                    for (int i = 0; i < VW; ++i) V::set(o, i, acc[k][i] - cmp[k][i]);
-                    V::stcs(orow + col.e[k], o);
-                }
+                        if (u < n && col.v[k]) V::stcs(orow + u * ostride + col.e[k], v[u][k]);
+                sx += kU4 * J;
+                orow += kU4 * ostride;
             }
         }
-        __syncwarp();
+        __syncwarp();   // s_x is reused by the next tile
+        t = t1;
+        r = r1;
+        t1 = t2;
+        r1 = r2;
+        q0 = q0n;
+        q1 = q1n;
+        id = idn;
+        q0n = q0m;
+        q1n = q1m;
     }
 }
 
@@ -494,28 +748,61 @@ size_t tile_smem(const TileGeom& g, const DevParams& p, size_t xbytes) {
     return sizeof(int64_t) * (size_t)(g.tb + 1) + xbytes * (size_t)g.qc * (size_t)p.J;
 }
 
-template <int VW, int KC, typename XT, bool SG>
-cudaError_t fwd_inst(const DevParams& p, const RowLayout& lay, const int64_t* idx, int64_t nnz,
+// Bags per tile of the forward: a multiple of the lane groups (and of 4), at
+// most kWarpPairs staged pairs and 16 bags or 4 per lane group, chosen so that
+// the warps' rounds of tiles waste least: rounds * (wb + 8) is smallest, a
+// tile's fixed work being about that of 8 bags.  Measured on GB300, us per
+// forward at 4, 8, 12, 16, 24 and 32 bags: Criteo-TB shape 227, 158, 150, 153,
+// 156, 156; multi-hot 326, 310, 303, 294, 298, 314; 16-float rows (batch 16384,
+// 8 lane groups) 36, 25, 18, 14, 11, 9.6.
+int tile_bags(const DevParams& p, const RowLayout& lay, int64_t rows, int64_t warps) {
+    const int ng = 32 >> lay.log2gs;
+    const int step = ng > 4 ? ng : 4;
+    int best = step;
+    int64_t best_cost = INT64_MAX;
+    const int most = 4 * ng > 16 ? 4 * ng : 16;
+    for (int wb = step; wb <= most; wb += step) {
+        if (wb > step && wb * p.J > kWarpPairs) break;
+        const int64_t tiles = (int64_t)p.T * ((rows + wb - 1) / wb);
+        const int64_t cost = ((tiles + warps - 1) / warps) * (wb + 8);
+        if (cost <= best_cost) {
+            best_cost = cost;
+            best = wb;
+        }
+    }
+    return best;
+}
+
+template <int VW, int KC, typename XT, bool SG, int MODE>
+cudaError_t fwd_mode(const DevParams& p, const RowLayout& lay, const int64_t* idx, int64_t nnz,
                      const int64_t* off, int64_t B, const float* w, float* out, DevError* err,
                      uint32_t* pair_x, uint32_t* q_row, int64_t b_lo, int64_t b_hi, int sm_count,
                      cudaStream_t st) {
-    // bags per warp tile: kU per lane group (kU loads in flight in the one-id
-    // path) and at least 16.  Measured on GB300: 16-bag tiles beat 32 and 64
-    // at the Criteo-TB shape (0.165 against 0.171 and 0.174 ms per forward)
-    // and on multi-id bags (0.385 against 0.419 ms), where the whole warp
-    // takes one bag at a time; the 16-float rows of the Criteo-Kaggle shape
-    // need the kU per group (batch 32768: 0.026 against 0.036 ms).
-    const int groups = 32 >> lay.log2gs;
-    const int wb = groups * kU > 16 ? groups * kU : 16;
-    const int tpt = (int)((b_hi - b_lo + wb - 1) / wb);
-    const size_t smem = (size_t)kWarps * ((size_t)(wb + 1) * sizeof(int64_t) +
-                                          (size_t)kWarpPairs * sizeof(XT));
+    const auto kern = k_forward_warp<VW, KC, XT, SG, MODE>;
+    const size_t smem = sizeof(XT) * (size_t)kWarps * (size_t)kWarpPairs;
+    const int64_t rows = b_hi - b_lo;
+    const int max_grid = grid_for(kern, sm_count, INT32_MAX, smem);
+    FwdGeom fg;
+    fg.wb = tile_bags(p, lay, rows, (int64_t)max_grid * kWarps);
+    fg.log2pw = ceil_log2(fg.wb);
+    fg.log2pi = 0;
+    while (fg.log2pi < 5 && (2 << fg.log2pi) * p.J <= kWarpPairs) ++fg.log2pi;
+    const int64_t tpt = (rows + fg.wb - 1) / fg.wb;
     const int64_t ntiles = (int64_t)p.T * tpt;
-    if (ntiles >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;
-    const int grid = grid_for(k_forward_warp<VW, KC, XT, SG>, sm_count, (ntiles + kWarps - 1) / kWarps,
-                              smem);
-    return launch_k(k_forward_warp<VW, KC, XT, SG>, dim3(grid), dim3(kThreads), smem, st, p, idx, nnz,
-                    off, B, w, out, err, pair_x, q_row, lay.log2gs, wb, tpt, b_lo, b_hi);
+    // (room for the stride past the last tile)
+    if (ntiles >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;
+    fg.tiles_per_table = (int)tpt;
+    fg.TJ = (uint64_t)p.T * (uint64_t)p.J;
+    fg.Gb = (uint64_t)p.G * sizeof(float);
+    for (int k = 0; k < 2; ++k) {
+        const unsigned lanes = 32u >> (k ? fg.log2pi : fg.log2pw);
+        fg.stepA[k] = (uint64_t)((unsigned __int128)p.A * lanes % kP61);
+        fg.stepA2[k] = (uint64_t)((unsigned __int128)p.A2 * lanes % kP61);
+    }
+    const int64_t blocks = (ntiles + kWarps - 1) / kWarps;
+    const int grid = blocks < max_grid ? (int)blocks : max_grid;
+    return launch_k(kern, dim3(grid), dim3(kThreads), smem, st, p, idx, nnz, off, B, w, out, err,
+                    pair_x, q_row, lay.log2gs, fg, b_lo, b_hi);
 }
 
 template <int VW, int KC, typename XT, typename AT, bool TOUCH>
@@ -530,20 +817,40 @@ cudaError_t sc_inst(const DevParams& p, const RowLayout& lay, const int64_t* idx
                     idx, nnz, off, B, gout, scale, target, tc, err, lay.log2gs, tg);
 }
 
+template <int VW, int KC, typename XT, bool SG>
+cudaError_t fwd_inst(const DevParams& p, const RowLayout& lay, const int64_t* idx, int64_t nnz,
+                     const int64_t* off, int64_t B, const float* w, float* out, DevError* err,
+                     uint32_t* pair_x, uint32_t* q_row, int64_t b_lo, int64_t b_hi, int sm_count,
+                     cudaStream_t st) {
+    // wider rows and 64-bit buckets have one variant
+    constexpr bool kModes = KC * VW <= 4 && sizeof(XT) == 4;
+    if (kModes && nnz > p.T * B)
+        return fwd_mode<VW, KC, XT, SG, kModes ? kFwdLong : kFwdShort>(
+            p, lay, idx, nnz, off, B, w, out, err, pair_x, q_row, b_lo, b_hi, sm_count, st);
+    // (8 rounds of 16 bags for the warps of 2 CTAs per SM)
+    if (kModes && lay.log2gs == 5 && p.T * (b_hi - b_lo) >= (int64_t)8 * 16 * 2 * kWarps * sm_count)
+        return fwd_mode<VW, KC, XT, SG, kModes ? kFwdMany : kFwdShort>(
+            p, lay, idx, nnz, off, B, w, out, err, pair_x, q_row, b_lo, b_hi, sm_count, st);
+    return fwd_mode<VW, KC, XT, SG, kFwdShort>(p, lay, idx, nnz, off, B, w, out, err, pair_x, q_row,
+                                               b_lo, b_hi, sm_count, st);
+}
+
 template <int VW, int KC>
 cudaError_t fwd_x(const DevParams& p, const RowLayout& lay, const int64_t* idx, int64_t nnz,
                   const int64_t* off, int64_t B, const float* w, float* out, DevError* err,
                   uint32_t* pair_x, uint32_t* q_row, int64_t b_lo, int64_t b_hi, int sm_count,
                   cudaStream_t st) {
-    if (p.R < 0xffffffffull)
+    // 32-bit buckets, and block starts below 2^32 bytes apart
+    if (p.R < 0xffffffffull && p.G < (int64_t(1) << 30))
         return p.smask ? fwd_inst<VW, KC, uint32_t, true>(p, lay, idx, nnz, off, B, w, out, err,
                                                            pair_x, q_row, b_lo, b_hi, sm_count, st)
                        : fwd_inst<VW, KC, uint32_t, false>(p, lay, idx, nnz, off, B, w, out, err,
                                                             pair_x, q_row, b_lo, b_hi, sm_count,
                                                             st);
-    // R >= 2^32: 64-bit buckets, never signed (signed hashing needs R < 2^31)
-    return fwd_inst<VW, KC, uint64_t, false>(p, lay, idx, nnz, off, B, w, out, err, nullptr,
-                                             nullptr, b_lo, b_hi, sm_count, st);
+    return p.smask ? fwd_inst<VW, KC, uint64_t, true>(p, lay, idx, nnz, off, B, w, out, err,
+                                                       pair_x, q_row, b_lo, b_hi, sm_count, st)
+                   : fwd_inst<VW, KC, uint64_t, false>(p, lay, idx, nnz, off, B, w, out, err,
+                                                        pair_x, q_row, b_lo, b_hi, sm_count, st);
 }
 
 template <int VW, int KC, typename AT>
