@@ -130,25 +130,35 @@ def _check(rc: int, what: str):
         raise PSSError(rc, what)
 
 
+_torch_mod = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_mod
+    if _torch_mod is None:
+        import torch
+        _torch_mod = torch
+    return _torch_mod
 
 
-def _stream_ptr(stream) -> ctypes.c_void_p:
+# The calls below are on the path of every step, and a small step's time is the
+# time of its calls: raw integers are passed for pointers (the argtypes convert
+# them), and the current stream's handle is read without building a Stream.
+def _stream_ptr(stream):
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _torch()
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(int(stream.cuda_stream))
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(int(t.data_ptr()))
+def _ptr(t) -> int:
+    return t.data_ptr()
 
 
 def _need(t, dtype, name):
-    torch = _torch()
-    if not isinstance(t, torch.Tensor):
+    if not isinstance(t, (_torch_mod or _torch()).Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
@@ -263,8 +273,8 @@ class PSS:
 
     def backward_update(self, grad_out, lr: float, stream=None):
         _need(grad_out, _torch().float32, "grad_out")
-        _check(self._lib.pss_backward_update(self._h, _ptr(grad_out), ctypes.c_float(lr),
-                                             _stream_ptr(stream)), "pss_backward_update")
+        _check(self._lib.pss_backward_update(self._h, _ptr(grad_out), lr, _stream_ptr(stream)),
+               "pss_backward_update")
 
     def backward_grad(self, grad_out, grad=None, stream=None):
         torch = _torch()

@@ -13,12 +13,14 @@ using namespace pss;
 
 namespace {
 
-// Restores the caller's current device on scope exit.
+// Makes `dev` current, and the caller's device again on scope exit (two calls
+// less where it is the current one already, as it nearly always is).
 struct DeviceGuard {
     int prev = -1;
-    bool ok = false;
     explicit DeviceGuard(int dev) {
-        if (cudaGetDevice(&prev) == cudaSuccess) ok = cudaSetDevice(dev) == cudaSuccess;
+        int cur = -1;
+        if (cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess)
+            prev = cur;
     }
     ~DeviceGuard() {
         if (prev >= 0) cudaSetDevice(prev);

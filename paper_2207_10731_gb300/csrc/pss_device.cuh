@@ -119,13 +119,45 @@ inline int ceil_log2(int v) {
     return l;
 }
 
+// CTAs of `threads` threads and `smem` bytes of dynamic shared memory (allowed
+// here where it is above the default 48 KB) that fit on an SM at once.  The
+// answer is a constant of the kernel and the device, and asking the runtime
+// costs about as much as a launch: each thread keeps what it was told.
+inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, int* per_sm) {
+    struct Known {
+        const void* kernel;
+        size_t smem;
+        int dev, threads, per_sm;
+    };
+    constexpr int kKnown = 64;
+    static thread_local Known known[kKnown] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const size_t h = ((size_t)kernel >> 4) * 0x9e3779b97f4a7c15ull + smem;
+    Known& k = known[(h >> 32) % kKnown];
+    if (k.kernel != kernel || k.smem != smem || k.dev != dev || k.threads != threads) {
+        if (smem > 48 * 1024) {
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) !=
+                cudaSuccess ||
+            n < 1)
+            n = 1;
+        k = Known{kernel, smem, dev, threads, n};
+    }
+    *per_sm = k.per_sm;
+    return cudaSuccess;
+}
+
 // Grid of a grid-stride kernel: all CTAs that fit at once, capped by the work.
 template <typename K>
 int grid_for(K kernel, int sm_count, int64_t work_blocks, size_t smem = 0) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreads, smem) !=
-            cudaSuccess ||
-        per_sm < 1)
+    int per_sm = 1;
+    if (resident_ctas(reinterpret_cast<const void*>(kernel), kThreads, smem, &per_sm) !=
+        cudaSuccess)
         per_sm = 1;
     int64_t g = (int64_t)sm_count * per_sm;
     if (work_blocks < g) g = work_blocks;

@@ -1458,8 +1458,9 @@ cudaError_t radix_pass(const SortedBuffers& sb, const unsigned long long* in,
                  st, sb.cnt, ntiles, bits, sb.tot, sb.dstart, sb.done, sb.stats);
     if (e != cudaSuccess) return e;
     const size_t smem = radix_down_smem(nd);
-    e = cudaFuncSetAttribute(k_radix_down<FIRST, SG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    int per_sm = 1;   // (allows the shared memory)
+    e = resident_ctas(reinterpret_cast<const void*>(k_radix_down<FIRST, SG>), kRThreads, smem,
+                      &per_sm);
     if (e != cudaSuccess) return e;
     return launch_k(k_radix_down<FIRST, SG>, dim3(ntiles), dim3(kRThreads), smem, st, sb.pair_x,
                     sb.q_row, in, out, npairs, sb.stats, J, log2J, shift, bits, ntiles, sb.cnt,
@@ -1601,13 +1602,10 @@ cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, ui
     const int log2J = ((J & (J - 1)) == 0) ? ceil_log2(J) : -1;
     const size_t smem = sizeof(uint32_t) * 2 * (size_t)kLSSlots;
     auto kern = smask ? k_sort_local<true> : k_sort_local<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    int per_sm = 1;
+    const cudaError_t e =
+        resident_ctas(reinterpret_cast<const void*>(kern), kLSThreads, smem, &per_sm);
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLSThreads, smem) !=
-            cudaSuccess || per_sm < 1)
-        per_sm = 1;
     const int64_t nseg = local_segments(npairs);
     const int grid = (int)(nseg < (int64_t)sm_count * per_sm ? nseg : (int64_t)sm_count * per_sm);
     return launch_k(kern, dim3(grid), dim3(kLSThreads), smem, st, sb.pair_x, npairs, sb.q_row, J,
