@@ -159,11 +159,12 @@ typedef enum {
      * runs of a location meet in the fp64 accumulator); no per-location
      * state, any R; needs chunks that tile the rows (Z = 32, d a multiple of
      * 32, 16-byte aligned upstream gradient), else the global sort runs.
-     * PSS_SORT_AUTO (default): local where it is served and either R > 2^22
-     * or the batch has at most PSS_SORT_LOCAL_MAX_PAIRS_PER_START pairs per
-     * block start (few repeats to merge across segments); global otherwise.
-     * After a local pass pss_info's last_collision_rate is -1 (no distinct
-     * locations are counted). */
+     * PSS_SORT_AUTO (default): where the local sort is served, local if R >
+     * 2^22 or the batch has at most PSS_SORT_LOCAL_MAX_PAIRS_PER_START pairs
+     * per block start; local with a count of the distinct locations above
+     * (bags of several ids: up to 30 pairs per start); global otherwise.
+     * pss_info's last_collision_rate is -1 after a local pass that did not
+     * count the distinct locations (PSS_SORT_LOCAL, or AUTO's first case). */
     PSS_OPT_SORT_SCOPE = 10
 } pss_option;
 

@@ -321,8 +321,10 @@ pss_status ensure_grad(pss_handle* h, cudaStream_t st) {
 // are allocated again on first use).  The caller has synchronised the device.
 void release_r_buffers(pss_handle* h) {
     for (void* b : {(void*)h->touched.bitmap, (void*)h->touched.list, (void*)h->touched.count,
-                    (void*)h->sb.ccnt, (void*)h->sb.start, (void*)h->sb.bsum, (void*)h->sb.bnz})
+                    (void*)h->sb.ccnt, (void*)h->sb.start, (void*)h->sb.bsum, (void*)h->sb.bnz,
+                    (void*)h->sb.seen})
         if (b) cudaFree(b);
+    h->sb.seen = nullptr;
     h->sb.ccnt = h->sb.start = h->sb.bsum = h->sb.bnz = nullptr;
     h->sb_counting = false;
     h->touched = Touched{};
@@ -646,7 +648,8 @@ pss_status pss_destroy(pss_handle* h) {
                     (void*)h->sb.tmp_e, (void*)h->sb.cnt, (void*)h->sb.tot,
                     (void*)h->sb.dstart, (void*)h->sb.done, (void*)h->sb.stats,
                     (void*)h->sb.ccnt, (void*)h->sb.start, (void*)h->sb.bsum,
-                    (void*)h->sb.bnz, (void*)h->sb.bnd, (void*)h->sb.segn})
+                    (void*)h->sb.bnz, (void*)h->sb.bnd, (void*)h->sb.segn,
+                    (void*)h->sb.seen})
         if (b) cudaFree(b);
     if (h->stats_host) cudaFreeHost(h->stats_host);
     if (h->stats_ev) cudaEventDestroy(h->stats_ev);
@@ -827,18 +830,68 @@ static pss_status scatter_into(pss_handle* h, const float* dgrad, float scale, f
                                       touch ? &h->touched : nullptr, h->err, h->sm_count, st));
 }
 
+// Bags of several ids: the sorted path reads a bag's gradient row once per id.
+static bool rows_reread(const pss_handle* h) { return h->last_nnz > h->dp.T * h->last_B; }
+
+// How the sorted path groups the pairs (PSS_OPT_SORT_SCOPE): within segments,
+// with or without a count of the distinct buckets, or all of them.
+enum LocalSort { kLocalNo, kLocalUncounted, kLocalCounted };
+
+// The local sort saves the global sort's per-bucket counters and atomics but
+// leaves one run per bucket and segment, each an fp64 reduction of a chunk
+// into g.  Measured on GB300 (us of sort + reduce, global against local, with
+// the count of distinct buckets where AUTO makes it):
+//   one id per bag: 0.1M pairs over 65K starts 36 / 33 (whole step), 6.8M over
+//   65K, 262K, 625K, 1M starts 271 / 238, 281 / 234, 285 / 239, 291 / 243;
+//   1.06M over 625K 66 / 48; 2^24 starts: radix 343 / 110 with the marking
+//   several ids per bag (Zipf 1.05, Zipf 1.2), by pairs per start:
+//   16: 476 / 465, 424 / 377     27 (Zipf 1.2): 414 / 377
+//   33: 465 / 468, 426 / 380     65: 449 / 459, 413 / 374
+//   130: 430 / 454, 386 / 367
+// The gradient of bags of several ids comes from L2, so runs cost more there
+// and the global sort's few runs win from about 30 pairs per start on.
+constexpr int64_t kLocalMaxRereadPairsPerStart = 30;
+
+static LocalSort use_local_sort(const pss_handle* h, int64_t npairs, bool touch,
+                                const float* dgrad) {
+    const int64_t R = (int64_t)h->dp.R;
+    if (h->deterministic || h->sort_scope == PSS_SORT_GLOBAL || !local_sort_ok(h->dp, dgrad))
+        return kLocalNo;
+    if (h->sort_scope == PSS_SORT_LOCAL || R > kCountSortMaxR ||
+        npairs <= (int64_t)PSS_SORT_LOCAL_MAX_PAIRS_PER_START * R)
+        return kLocalUncounted;
+    // (the touched list of a counted batch comes from the counting sort's scan)
+    if (touch || (rows_reread(h) && npairs > kLocalMaxRereadPairsPerStart * R)) return kLocalNo;
+    return kLocalCounted;
+}
+
+// The byte per bucket of a local sort that counts (zero between sorts: zeroed
+// here, and by every reduce that has counted it).
+static pss_status ensure_seen(pss_handle* h, cudaStream_t st) {
+    if (h->sb.seen) return PSS_OK;
+    const size_t bytes = ((size_t)h->dp.R + 15) / 16 * 16;
+    PSS_TRY(cudaMalloc(&h->sb.seen, bytes));
+    PSS_TRY(cudaMemsetAsync(h->sb.seen, 0, bytes, st));
+    return PSS_OK;
+}
+
 // Sorted path, step 1: sort the last forward's pairs by bucket (counting or
 // radix sort); with `touch`, also list the touched blocks.
-static pss_status sort_pairs(pss_handle* h, bool touch, bool local, cudaStream_t st) {
+static pss_status sort_pairs(pss_handle* h, bool touch, LocalSort local, cudaStream_t st) {
     const int64_t npairs = h->last_nnz * (int64_t)h->dp.J;
     poll_stats(h);
-    if (local) {
-        // grouped within segments only: no global count of distinct buckets
-        LaunchScope ls(h, PSS_K_SORT, st, touch ? 2 : 1);
-        PSS_TRY(launch_sort_local(h->sb, npairs, h->dp.J, h->dp.smask, h->sm_count, st));
-        if (touch)
-            PSS_TRY(launch_mark_pairs(h->sb, npairs, h->dp.smask, h->touched, h->sm_count, st));
-        h->last_collision = -1.0;
+    if (local != kLocalNo) {
+        // grouped within segments only: the distinct buckets are marked and
+        // counted where the collision rate is reported
+        if (local == kLocalCounted) {
+            pss_status rc0 = ensure_seen(h, st);
+            if (rc0 != PSS_OK) return rc0;
+        } else {
+            h->last_collision = -1.0;
+        }
+        LaunchScope ls(h, PSS_K_SORT, st, 1);
+        PSS_TRY(launch_sort_local(h->sb, npairs, h->dp.J, h->dp.smask,
+                                  touch ? &h->touched : nullptr, h->sm_count, st));
     } else if (use_radix(h)) {
         pss_status rc0 = ensure_radix(h, npairs, st);
         if (rc0 != PSS_OK) return rc0;
@@ -872,9 +925,6 @@ static pss_status copy_stats(pss_handle* h, cudaStream_t st) {
     return PSS_OK;
 }
 
-// Bags of several ids: the sorted path reads a bag's gradient row once per id.
-static bool rows_reread(const pss_handle* h) { return h->last_nnz > h->dp.T * h->last_B; }
-
 // Sorted path with the window reduce: sort (with `touch`, also list the
 // touched blocks), then every element's gradient stored once into gexp
 // (fp32, zero on entry).
@@ -882,7 +932,7 @@ static pss_status sorted_window(pss_handle* h, const float* dgrad, bool staged, 
                                 float* gexp, cudaStream_t st) {
     const int64_t npairs = h->last_nnz * (int64_t)h->dp.J;
     if (h->dp.T * h->last_B == 0 || npairs == 0) return grad_wait(h, staged, st);
-    pss_status rc = sort_pairs(h, touch, false, st);
+    pss_status rc = sort_pairs(h, touch, kLocalNo, st);
     if (rc != PSS_OK) return rc;
     if ((rc = grad_wait(h, staged, st)) != PSS_OK) return rc;
     {
@@ -902,30 +952,13 @@ static pss_status ensure_g32(pss_handle* h, cudaStream_t st) {
     return PSS_OK;
 }
 
-// Segment-local or global sort (PSS_OPT_SORT_SCOPE).  The local sort saves
-// the global sort's per-bucket counters and atomics but leaves one run per
-// bucket and segment, each an fp64 reduction of a chunk into g: it pays
-// where few pairs share a block start, and above 2^22 starts, where the
-// global sort is the radix sort.  Measured on GB300 (ms per step, global
-// against local): Criteo-TB shape at 1.4, 2.7, 4.1 and 11 pairs per start
-// 0.098/0.090, 0.152/0.153, 0.207/0.215, 0.465/0.495; paper micro-benchmark
-// shape (1.7) 0.110/0.105; M = 2^22 at 3.3 per start 0.275/0.274; M = 2^24
-// (1.6) 0.635/0.629; M = 2^28 (radix) 1.31/1.20.
-static bool use_local_sort(const pss_handle* h, int64_t npairs, const float* dgrad) {
-    if (h->deterministic || h->sort_scope == PSS_SORT_GLOBAL || !local_sort_ok(h->dp, dgrad))
-        return false;
-    if (h->sort_scope == PSS_SORT_LOCAL) return true;
-    return (int64_t)h->dp.R > kCountSortMaxR ||
-           npairs <= (int64_t)PSS_SORT_LOCAL_MAX_PAIRS_PER_START * (int64_t)h->dp.R;
-}
-
 // Sorted path: sort by bucket (segment-local, counting or radix), segmented
 // reduce into g64.
 static pss_status sorted_into64(pss_handle* h, const float* dgrad, bool staged, bool touch,
                                 cudaStream_t st) {
     const int64_t npairs = h->last_nnz * (int64_t)h->dp.J;
     if (h->dp.T * h->last_B == 0 || npairs == 0) return PSS_OK;
-    const bool local = use_local_sort(h, npairs, dgrad);
+    const LocalSort local = use_local_sort(h, npairs, touch, dgrad);
     pss_status rc0 = sort_pairs(h, touch, local, st);
     if (rc0 != PSS_OK) return rc0;
     // the sort above needs only the forward's buckets: a host gradient's copy
@@ -934,10 +967,17 @@ static pss_status sorted_into64(pss_handle* h, const float* dgrad, bool staged, 
     if (rc != PSS_OK) return rc;
     {
         LaunchScope ls(h, PSS_K_REDUCE, st);
-        PSS_TRY(launch_sorted_reduce(h->sb, npairs, dgrad, h->dp, h->g64, local,
-                                     !local && use_radix(h), rows_reread(h), h->sm_count, st));
+        PSS_TRY(launch_sorted_reduce(h->sb, npairs, dgrad, h->dp, h->g64, local != kLocalNo,
+                                     local == kLocalNo && use_radix(h), rows_reread(h),
+                                     local == kLocalCounted ? h->sb.seen : nullptr, h->sm_count,
+                                     st));
     }
-    return local ? PSS_OK : copy_stats(h, st);
+    if (local == kLocalUncounted) return PSS_OK;
+    if (local == kLocalCounted) {
+        LaunchScope ls(h, PSS_K_MISC, st);
+        PSS_TRY(launch_count_seen(h->sb, npairs, (int64_t)h->dp.R, h->sm_count, st));
+    }
+    return copy_stats(h, st);
 }
 
 pss_status pss_backward_update(pss_handle* h, const float* grad_out, float lr, pss_stream stream) {

@@ -86,6 +86,7 @@ struct SortedBuffers {
     unsigned long long* stats;    // [0] valid pairs, [1] distinct buckets
     float* bnd;                   // window reduce: boundary records, 64 floats per range
     uint32_t* segn;               // local sort: valid pairs of each segment
+    uint8_t* seen;                // local sort: 1 per bucket in the batch (zero between sorts)
     // counting sort (R <= kCountSortMaxR)
     uint32_t* ccnt;               // R counts per bucket (zero between sorts)
     uint32_t* start;              // R + 1 bucket starts
@@ -124,16 +125,22 @@ cudaError_t launch_mark_pairs(const SortedBuffers& sb, int64_t npairs, uint32_t 
 // staged reduce (local_sort_ok) with R < 2^32 - 1; any R, no per-bucket state.
 int64_t local_segments(int64_t npairs);
 bool local_sort_ok(const DevParams& p, const float* gout);
+// With `touched`, also the touched bitmap and list of the buckets.
 cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
-                              int sm_count, cudaStream_t st);
+                              const Touched* touched, int sm_count, cudaStream_t st);
+// Adds the valid pairs and the distinct buckets that a reduce marked in sb.seen
+// to stats (zero on entry), and clears the marks.
+cudaError_t launch_count_seen(const SortedBuffers& sb, int64_t npairs, int64_t R, int sm_count,
+                              cudaStream_t st);
 // Reduce of the sorted entries into g (fp64).  `local`: the entries come from
 // the segment-local sort (one run per bucket and segment).  `count_runs`: the
 // reduce counts the distinct buckets into stats[1] (the radix sort's entries;
 // the counting sort's scan counts them itself).  `reread`: the gradient's rows
-// are read several times (bags of several ids), so they are kept in L2.
+// are read several times (bags of several ids), so they are kept in L2.  `seen`
+// (local only, may be null): the buckets with entries are marked there.
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
-                                 bool reread, int sm_count, cudaStream_t st);
+                                 bool reread, uint8_t* seen, int sm_count, cudaStream_t st);
 // Window reduce (see pss_sorted.cu): run sums go into each task's sliding
 // element window; every element's gradient is stored once into gexp (fp32,
 // zero where the batch adds nothing; the caller zero-fills it), in a fixed

@@ -321,106 +321,145 @@ k_sort_scatter(const uint32_t* __restrict__ pair_x, int64_t npairs, const uint32
 // so a segment merges the repeats of the table's hot ids (under Zipf ids the
 // ones that would otherwise queue reductions on one address).
 //
-// Within a segment: every thread inserts its pairs into a shared-memory hash
-// table (bucket -> count; each pair's rank among the segment's pairs of its
-// bucket), the slot counts are scanned in a fixed slot order, and a pair goes
-// to its slot's start plus its rank.  Which pair of a bucket comes first
-// follows the order of the shared-memory atomics.
+// Within a segment: a pair's SLOT is the top bits of a multiplicative hash of
+// its bucket; one returning shared-memory atomic on the slot's 16-bit counter
+// gives its rank, the counters are scanned in a fixed slot order, and a pair
+// goes to its slot's start plus its rank.  Buckets are not compared: two that
+// share a slot interleave there, which only splits their runs (at Criteo-TB
+// about 3300 buckets of a segment meet in 32768 slots).  Which pair of a slot
+// comes first follows the order of the shared-memory atomics.
+// What bounds it: the latency of a segment's phases (load, rank, scan, place,
+// write).  So the entries are placed in the counters' own shared memory once
+// every place is known, and two CTAs of 1024 threads share an SM.  Measured on
+// GB300: 41 us at the Criteo-TB shape (6.8M pairs), 9.2 us at the
+// micro-benchmark's (1.06M), against 64 and 12.7 us with a hash table of keys
+// and counts (128 KB, one CTA per SM, a compare-and-swap per pair).
 constexpr int kLSLog2 = 13;
 constexpr int kLS = 1 << kLSLog2;                 // pairs per segment (8192)
 constexpr int kLSThreads = 1024;
 constexpr int kLSPer = kLS / kLSThreads;          // pairs per thread
-constexpr int kLSLog2Slots = kLSLog2 + 1;         // load factor <= 1/2
-constexpr int kLSSlots = 1 << kLSLog2Slots;
-constexpr int kLSSlotsPer = kLSSlots / kLSThreads;
-static_assert(kLS <= 65536 && kLSSlots <= 65536, "slot and rank are packed in 16 bits each");
+constexpr int kLSLog2Slots = 15;
+constexpr int kLSWords = (1 << kLSLog2Slots) / 2; // two counters per word
+constexpr int kLSOwn = kLSWords / kLSThreads;     // words per thread
+static_assert(kLS < 65536, "counters, ranks and places are 16-bit");
+static_assert(kLSWords * 4 == kLS * 8, "the entries take the counters' place");
 static_assert(kLSThreads == kScanThreads, "the local sort scans with block_exclusive_scan");
 
-__device__ __forceinline__ uint32_t local_insert(uint32_t* s_key, uint32_t* s_val, uint32_t x) {
-    uint32_t h = (x * 0x9e3779b1u) >> (32 - kLSLog2Slots);
-    for (int probe = 0; probe < kLSSlots; ++probe) {
-        const uint32_t prev = atomicCAS(s_key + h, kEmpty, x);
-        if (prev == kEmpty || prev == x) break;
-        h = (h + 1u) & (uint32_t)(kLSSlots - 1);
-    }
-    return h | (atomicAdd(s_val + h, 1u) << 16);
+// With TOUCH, a segment's distinct buckets also enter the touched bitmap and list.
+__host__ __device__ constexpr size_t local_smem(bool touch) {
+    return sizeof(unsigned long long) * kLS + (touch ? sizeof(uint32_t) * kLS : 0);
 }
 
 // sorted_e[s*kLS + pos] = x << 32 | row*J + j for the valid pairs of segment
-// s, grouped by x; segn[s] = the segment's number of valid pairs.
-template <bool SG>
-__global__ void __launch_bounds__(kLSThreads, 1)
+// s, grouped by x; segn[s] = the segment's number of valid pairs; stats = {0, 0}
+// (k_count_seen adds to them).
+template <bool SG, bool TOUCH>
+__global__ void __launch_bounds__(kLSThreads, 2)
 k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
              const uint32_t* __restrict__ q_row, int J, int log2J,
-             unsigned long long* __restrict__ sorted_e, uint32_t* __restrict__ segn) {
+             unsigned long long* __restrict__ sorted_e, uint32_t* __restrict__ segn,
+             Touched tc, unsigned long long* __restrict__ stats) {
     pdl_prologue();
-    extern __shared__ __align__(16) uint32_t s_ls[];
-    uint32_t* s_key = s_ls;
-    uint32_t* s_val = s_ls + kLSSlots;
+    extern __shared__ __align__(16) unsigned char ls_smem[];
+    uint32_t* s_w = reinterpret_cast<uint32_t*>(ls_smem);                               // [kLSWords]
+    unsigned long long* s_e = reinterpret_cast<unsigned long long*>(ls_smem);           // [kLS]
+    uint32_t* s_new = reinterpret_cast<uint32_t*>(ls_smem + sizeof(unsigned long long) * kLS);
     __shared__ uint32_t s_warp[33];
+    __shared__ uint32_t s_n;
+    __shared__ unsigned long long s_base;
     const int tid = threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < kLSSlotsPer; ++k) {
-        s_key[k * kLSThreads + tid] = kEmpty;
-        s_val[k * kLSThreads + tid] = 0u;
-    }
+    if (blockIdx.x == 0 && tid < 2) stats[tid] = 0ull;
     const int64_t nseg = (npairs + kLS - 1) / kLS;
     for (int64_t seg = blockIdx.x; seg < nseg; seg += gridDim.x) {
         const int64_t p0 = seg * kLS;
-        uint32_t x[kLSPer], e[kLSPer], hr[kLSPer];
+        uint32_t x[kLSPer];
 #pragma unroll
         for (int i = 0; i < kLSPer; ++i) {
             const int64_t p = p0 + i * kLSThreads + tid;
             x[i] = (p < npairs) ? __ldg(pair_x + p) : kBad;
         }
 #pragma unroll
-        for (int i = 0; i < kLSPer; ++i) {
-            const uint32_t pp = (uint32_t)(p0 + i * kLSThreads + tid);   // npairs < 2^32 here
-            const uint32_t q = (log2J >= 0) ? (pp >> log2J) : pp / (uint32_t)J;
-            e[i] = pp - q * (uint32_t)J;
-            if (x[i] != kBad) {
-                e[i] += __ldg(q_row + q) * (uint32_t)J;
-                if (SG) {
-                    // signed hashing: the sign moves to bit 31 of the entry's low word
-                    e[i] |= x[i] & 0x80000000u;
-                    x[i] &= 0x7fffffffu;
-                }
-            }
-        }
-        __syncthreads();   // the previous segment's table is clear
-#pragma unroll
-        for (int i = 0; i < kLSPer; ++i)
-            hr[i] = (x[i] != kBad) ? local_insert(s_key, s_val, x[i]) : 0u;
+        for (int k = 0; k < kLSWords / 4 / kLSThreads; ++k)
+            reinterpret_cast<uint4*>(s_w)[k * kLSThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+        if (TOUCH && tid == 0) s_n = 0u;
         __syncthreads();
-        // slot starts: exclusive prefix of the counts in the order (thread,
-        // k) over the slots tid + k*kLSThreads that thread tid owns
-        uint32_t c[kLSSlotsPer], own = 0u;
+        auto slot_of = [](uint32_t xi) {
+            return ((SG ? xi & 0x7fffffffu : xi) * 0x9e3779b1u) >> (32 - kLSLog2Slots);
+        };
+        uint32_t pos[kLSPer];
 #pragma unroll
-        for (int k = 0; k < kLSSlotsPer; ++k) {
-            c[k] = s_val[k * kLSThreads + tid];
-            own += c[k];
+        for (int i = 0; i < kLSPer; ++i) {
+            const uint32_t sl = slot_of(x[i]), sh = (sl & 1u) * 16u;
+            pos[i] = (x[i] != kBad) ? (atomicAdd(s_w + (sl >> 1), 1u << sh) >> sh) & 0xffffu : 0u;
+        }
+        __syncthreads();
+        // slot starts: exclusive prefix of the counts in the order (thread, k)
+        // over the words tid + k*kLSThreads that thread tid owns
+        uint32_t own = 0u;
+#pragma unroll
+        for (int k = 0; k < kLSOwn; ++k) {
+            const uint32_t c = s_w[k * kLSThreads + tid];
+            own += (c & 0xffffu) + (c >> 16);
         }
         uint32_t total;
         uint32_t run = block_exclusive_scan(own, s_warp, &total);
 #pragma unroll
-        for (int k = 0; k < kLSSlotsPer; ++k) {
-            s_val[k * kLSThreads + tid] = run;
-            run += c[k];
+        for (int k = 0; k < kLSOwn; ++k) {
+            const uint32_t c = s_w[k * kLSThreads + tid];
+            const uint32_t mid = run + (c & 0xffffu);
+            s_w[k * kLSThreads + tid] = run | mid << 16;   // (kLS itself only past the last pair)
+            run = mid + (c >> 16);
+        }
+        // entries: row*J + j of the pair (loads in flight during the scan)
+        uint32_t e[kLSPer];
+#pragma unroll
+        for (int i = 0; i < kLSPer; ++i) {
+            const uint32_t pp = (uint32_t)(p0 + i * kLSThreads + tid);   // npairs < 2^32 here
+            const uint32_t q = (log2J >= 0) ? (pp >> log2J) : pp / (uint32_t)J;
+            e[i] = pp - q * (uint32_t)J;
+            if (x[i] != kBad) e[i] += __ldg(q_row + q) * (uint32_t)J;
         }
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < kLSPer; ++i) {
+            const uint32_t sl = slot_of(x[i]);
+            pos[i] += (s_w[sl >> 1] >> ((sl & 1u) * 16u)) & 0xffffu;
+        }
+        __syncthreads();   // every place is known: the entries take the counters' place
+#pragma unroll
+        for (int i = 0; i < kLSPer; ++i) {
             if (x[i] == kBad) continue;
-            const uint32_t pos = s_val[hr[i] & 0xffffu] + (hr[i] >> 16);
-            sorted_e[p0 + pos] = ((unsigned long long)x[i] << 32) | e[i];
+            // signed hashing: the sign moves to bit 31 of the entry's low word
+            const uint32_t xi = SG ? x[i] & 0x7fffffffu : x[i];
+            const uint32_t ei = SG ? e[i] | (x[i] & 0x80000000u) : e[i];
+            s_e[pos[i]] = ((unsigned long long)xi << 32) | ei;
         }
         if (tid == 0) segn[seg] = total;
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < kLSSlotsPer; ++k) {
-            s_key[k * kLSThreads + tid] = kEmpty;
-            s_val[k * kLSThreads + tid] = 0u;
+        for (int i = 0; i < kLSPer; ++i) {
+            const uint32_t l = i * kLSThreads + tid;
+            if (l >= total) break;
+            const unsigned long long v = s_e[l];
+            sorted_e[p0 + l] = v;
+            if (TOUCH) {
+                const uint32_t xi = (uint32_t)(v >> 32), bit = 1u << (xi & 31u);
+                if ((l == 0 || (uint32_t)(s_e[l - 1] >> 32) != xi) &&   // a run's first entry
+                    !(atomicOr(tc.bitmap + (xi >> 5), bit) & bit))
+                    s_new[atomicAdd(&s_n, 1u)] = xi;
+            }
         }
+        if (TOUCH) {   // one reservation of list places per segment
+            __syncthreads();
+            const uint32_t n = s_n;
+            if (tid == 0) s_base = n ? atomicAdd(tc.count, (unsigned long long)n) : 0ull;
+            __syncthreads();
+            for (uint32_t k = tid; k < n; k += kLSThreads) {
+                const unsigned long long slot = s_base + k;
+                if ((int64_t)slot < tc.cap) tc.list[slot] = (int64_t)s_new[k];
+            }
+        }
+        __syncthreads();   // the shared memory is used again
     }
 }
 
@@ -1119,7 +1158,8 @@ __global__ void __launch_bounds__(kThreads, 4)
 k_async_reduce(const unsigned long long* __restrict__ sorted_e,
                unsigned long long* __restrict__ stats, int64_t npairs, int64_t per,
                const float* __restrict__ gout, bool reread, uint32_t G, double* __restrict__ g,
-               WindowSink ws, const uint32_t* __restrict__ segn, bool count_runs) {
+               WindowSink ws, const uint32_t* __restrict__ segn, bool count_runs,
+               uint8_t* __restrict__ seen) {
     pdl_prologue();
     __shared__ __align__(16) float s_ring[kWarps][kAD][kAS][32];
     const int64_t total =
@@ -1240,6 +1280,9 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
         uint32_t xp = __shfl_up_sync(0xffffffffu, x0, 1);
         if (lane == 0) xp = xlast;
         const uint32_t heads = __ballot_sync(0xffffffffu, x0 != xp);
+        // (the range's first entry is not a head: its run may go on from the
+        // range before)
+        if (LOCAL && seen && x0 != kBad && (x0 != xp || (k == 0 && lane == 0))) seen[x0] = 1;
         xlast = __shfl_sync(0xffffffffu, x0, 31);
         if (!LOCAL && count_runs)
             nstart += __popc(heads & __ballot_sync(0xffffffffu, x0 != kBad));
@@ -1292,6 +1335,32 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
     // (the local layout's runs are per segment: no distinct-bucket count)
     if (!LOCAL && count_runs && lane == 0 && nstart)
         atomicAdd(stats + 1, (unsigned long long)nstart);
+}
+
+// After a reduce that marked its buckets: valid pairs and distinct buckets are
+// added to stats (zero on entry), and the marks return to zero.
+__global__ void __launch_bounds__(kThreads)
+k_count_seen(const uint32_t* __restrict__ segn, int64_t nseg, uint8_t* __restrict__ seen,
+             int64_t n16, unsigned long long* __restrict__ stats) {
+    pdl_prologue();
+    uint32_t valid = 0u, distinct = 0u;
+    uint4* seen4 = reinterpret_cast<uint4*>(seen);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nseg || i < n16;
+         i += stride) {
+        if (i < nseg) valid += __ldg(segn + i);
+        if (i < n16) {
+            const uint4 w = seen4[i];   // 16 buckets, 0 or 1 each
+            distinct += __popc(w.x) + __popc(w.y) + __popc(w.z) + __popc(w.w);
+            if (w.x | w.y | w.z | w.w) seen4[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
+    valid = __reduce_add_sync(0xffffffffu, valid);
+    distinct = __reduce_add_sync(0xffffffffu, distinct);
+    if ((threadIdx.x & 31) == 0) {
+        if (valid) atomicAdd(stats, (unsigned long long)valid);
+        if (distinct) atomicAdd(stats + 1, (unsigned long long)distinct);
+    }
 }
 
 // The boundary elements of the window reduce.  Between task j - 1 and task j
@@ -1534,20 +1603,24 @@ bool window_reduce_ok(const DevParams& p, const float* gout) {
 }
 
 // CTAs of the staged reduce per SM (at most 4 are resident; more give the
-// hardware ranges to balance with).  Measured on GB300, us per reduce:
-//                                   2      3      4      8     12
-//   global sort, rows read once   164    183    192    187    180   (Criteo-TB)
-//   global sort, rows re-read     245    200    195    190    190   (multi-hot)
-//   local sort                   43.1   44.4   44.0   41.7   42.2   (micro-benchmark)
-//                                99.9   99.1   96.6   90.8   89.0   (M = 2^26, batch 16384)
-//   window (deterministic)       95.6   79.7   77.9   77.7          (batch 20011), and its
-//   combine                       4.9    6.2    6.7   11.4
+// hardware ranges to balance with, and keep the ranges in work close together).
+// Measured on GB300, us per reduce:
+//                                   2     3     4     8    12    16    32    64
+//   global sort, rows read once   164   183   192   187   180   ---   ---   ---  (Criteo-TB)
+//   global sort, rows re-read     245   200   195   190   190   ---   ---   ---  (multi-hot)
+//   local sort, rows read once    224   219   223   210   199   198   187   184  (Criteo-TB)
+//                                43.1  44.7  44.4  42.1  41.7  39.7  39.9  39.8  (micro)
+//                                99.9   100  97.1  90.2  88.5  88.3  87.2  87.7  (M = 2^26)
+//   local sort, rows re-read      365   304   280   284   274   273   271   282  (multi-hot)
+//   window (deterministic)       95.6  79.7  77.9  77.7              (batch 20011), and its
+//   combine                       4.9   6.2   6.7  11.4
 // Rows read once in bucket order are random 128-byte HBM reads, of which fewer
-// in flight are served faster; the others wait for L2 and the reductions.
+// in flight are served faster.  A local sort's ranges in order walk through
+// the gradient's rows, so small ranges read rows that lie together.
 constexpr int kWindowCtas = 3;
 static int staged_ctas(int sink, bool local, bool reread) {
     if (sink == kSinkOnce) return kWindowCtas;
-    return local || reread ? 8 : 2;
+    return local ? 32 : reread ? 8 : 2;
 }
 
 // Entries per warp of the staged reduce over `entries` sorted entries.
@@ -1569,13 +1642,13 @@ template <int SINK, bool LOCAL>
 static cudaError_t staged_reduce(const SortedBuffers& sb, int64_t npairs, int64_t entries,
                                  const float* gout, bool reread, const DevParams& p, double* g,
                                  const WindowSink& ws, const uint32_t* segn, bool count_runs,
-                                 int sm_count, cudaStream_t st) {
+                                 uint8_t* seen, int sm_count, cudaStream_t st) {
     const int64_t per = staged_per(entries, staged_ctas(SINK, LOCAL, reread), sm_count);
     const int64_t tasks = (entries + per - 1) / per;
     const int grid = (int)((tasks + kWarps - 1) / kWarps);
     auto kern = p.smask ? k_async_reduce<SINK, LOCAL, true> : k_async_reduce<SINK, LOCAL, false>;
     return launch_k(kern, dim3(grid), dim3(kThreads), 0, st, sb.sorted_e, sb.stats, npairs, per,
-                    gout, reread, (uint32_t)p.G, g, ws, segn, count_runs);
+                    gout, reread, (uint32_t)p.G, g, ws, segn, count_runs, seen);
 }
 
 cudaError_t launch_window_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
@@ -1583,7 +1656,7 @@ cudaError_t launch_window_reduce(const SortedBuffers& sb, int64_t npairs, const 
                                  int sm_count, cudaStream_t st) {
     if (!window_reduce_ok(p, gout)) return cudaErrorInvalidValue;
     const cudaError_t e = staged_reduce<kSinkOnce, false>(sb, npairs, npairs, gout, reread, p,
-                                                          nullptr, ws, nullptr, true, sm_count, st);
+                                                          nullptr, ws, nullptr, true, nullptr, sm_count, st);
     if (e != cudaSuccess) return e;
     const int64_t per = staged_per(npairs, kWindowCtas, sm_count);
     const int64_t ntasks = (npairs + per - 1) / per;   // upper bound
@@ -1597,33 +1670,44 @@ int64_t local_segments(int64_t npairs) { return (npairs + kLS - 1) / kLS; }
 bool local_sort_ok(const DevParams& p, const float* gout) { return window_reduce_ok(p, gout); }
 
 cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
-                              int sm_count, cudaStream_t st) {
+                              const Touched* touched, int sm_count, cudaStream_t st) {
     if (npairs <= 0) return cudaSuccess;
     const int log2J = ((J & (J - 1)) == 0) ? ceil_log2(J) : -1;
-    const size_t smem = sizeof(uint32_t) * 2 * (size_t)kLSSlots;
-    auto kern = smask ? k_sort_local<true> : k_sort_local<false>;
+    const auto kern = smask ? (touched ? k_sort_local<true, true> : k_sort_local<true, false>)
+                            : (touched ? k_sort_local<false, true> : k_sort_local<false, false>);
+    const size_t smem = local_smem(touched != nullptr);
     int per_sm = 1;
     const cudaError_t e =
         resident_ctas(reinterpret_cast<const void*>(kern), kLSThreads, smem, &per_sm);
     if (e != cudaSuccess) return e;
-    const int64_t nseg = local_segments(npairs);
-    const int grid = (int)(nseg < (int64_t)sm_count * per_sm ? nseg : (int64_t)sm_count * per_sm);
-    return launch_k(kern, dim3(grid), dim3(kLSThreads), smem, st, sb.pair_x, npairs, sb.q_row, J,
-                    log2J, sb.sorted_e, sb.segn);
+    const int64_t nseg = local_segments(npairs), most = (int64_t)sm_count * per_sm;
+    return launch_k(kern, dim3((unsigned)(nseg < most ? nseg : most)), dim3(kLSThreads), smem, st,
+                    sb.pair_x, npairs, sb.q_row, J, log2J, sb.sorted_e, sb.segn,
+                    touched ? *touched : Touched{}, sb.stats);
+}
+
+cudaError_t launch_count_seen(const SortedBuffers& sb, int64_t npairs, int64_t R, int sm_count,
+                              cudaStream_t st) {
+    const int64_t n16 = (R + 15) / 16, nseg = local_segments(npairs);
+    const int64_t work = n16 > nseg ? n16 : nseg;
+    const int grid = grid_for(k_count_seen, sm_count, (work + kThreads - 1) / kThreads);
+    return launch_k(k_count_seen, dim3(grid), dim3(kThreads), 0, st, sb.segn, nseg, sb.seen, n16,
+                    sb.stats);
 }
 
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
-                                 bool reread, int sm_count, cudaStream_t st) {
+                                 bool reread, uint8_t* seen, int sm_count, cudaStream_t st) {
     if (local && !window_reduce_ok(p, gout)) return cudaErrorInvalidValue;
     // 32-element chunks tiling the rows: asynchronous shared-memory staging
     if (window_reduce_ok(p, gout)) {
         if (local)
             return staged_reduce<kSinkF64, true>(sb, npairs, local_segments(npairs) * kLS, gout,
-                                                 reread, p, g, WindowSink{}, sb.segn, false,
+                                                 reread, p, g, WindowSink{}, sb.segn, false, seen,
                                                  sm_count, st);
         return staged_reduce<kSinkF64, false>(sb, npairs, npairs, gout, reread, p, g, WindowSink{},
-                                              nullptr, count_runs, sm_count, st);
+                                              nullptr, count_runs, nullptr, sm_count,
+                                              st);
     }
     // blocks of 32+ elements: one warp per task, one element per lane
     if (p.L >= 32) {
