@@ -90,9 +90,11 @@ typedef enum {
      * accumulation bound; dyadic inputs give identical bits).  The sorted path
      * groups the contributions by location and sums each location's run once
      * (see PSS_OPT_DETERMINISTIC for its order).  PSS_PATH_AUTO takes the
-     * sorted path when the batch adds at least 5,000,000 elements (nnz * J *
-     * L) with blocks of L >= 32 elements, 10,000,000 with shorter blocks, the
-     * atomic one below (crossovers measured on GB300; M does not move them). */
+     * sorted path when the batch adds at least 3,500,000 elements (nnz * J *
+     * L) where the local sort serves it (PSS_OPT_SORT_SCOPE; blocks of L >= 8
+     * elements, fp64 accumulation); otherwise 5,000,000 with blocks of L >= 32
+     * elements and 10,000,000 with shorter ones; the atomic one below
+     * (crossovers measured on GB300; M does not move them). */
     PSS_OPT_BACKWARD_PATH = 1,
     /* How the Adagrad step visits M: every element (PSS_UPDATE_DENSE), only the
      * blocks the batch touched (PSS_UPDATE_TOUCHED), or chosen from M and the
@@ -158,13 +160,19 @@ typedef enum {
      * of 8192 consecutive pairs only, one run per location and segment (the
      * runs of a location meet in the fp64 accumulator); no per-location
      * state, any R; needs chunks that tile the rows (Z = 32, d a multiple of
-     * 32, 16-byte aligned upstream gradient), else the global sort runs.
+     * 32, 16-byte aligned upstream gradient).  Other chunk shapes are grouped
+     * within segments too, with the distinct locations counted, where R <=
+     * 2^22, the update is the dense one, the batch is one that PSS_PATH_AUTO
+     * would sort, and L is 4, 8 or 16 (chunks that tile the rows) or 32 to 128;
+     * else the global sort runs.
      * PSS_SORT_AUTO (default): where the local sort is served, local if R >
      * 2^22 or the batch has at most PSS_SORT_LOCAL_MAX_PAIRS_PER_START pairs
      * per block start; local with a count of the distinct locations above
-     * (bags of several ids: up to 30 pairs per start); global otherwise.
+     * (bags of several ids: up to 30 pairs per start) and for the other chunk
+     * shapes named above; global otherwise.
      * pss_info's last_collision_rate is -1 after a local pass that did not
-     * count the distinct locations (PSS_SORT_LOCAL, or AUTO's first case). */
+     * count the distinct locations (Z = 32 with PSS_SORT_LOCAL, or with AUTO's
+     * first case). */
     PSS_OPT_SORT_SCOPE = 10
 } pss_option;
 

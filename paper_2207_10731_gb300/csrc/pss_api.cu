@@ -389,17 +389,30 @@ bool use_touched(const pss_handle* h, int64_t pairs) {
 // The sorted path holds bucket indices in 32 bits, 0xffffffff marking a bad
 // id: it needs R < kSortedMaxR, the bound below which the forward emits 32-bit
 // buckets at all.  AUTO takes the sorted path when the batch adds at least
-// auto_sorted_min_adds(L) elements (pairs * L), the atomic path below: the
+// auto_sorted_min_adds elements (pairs * L), the atomic path below: the
 // atomic path's one kernel wins small batches, the sorted path's sort and
 // reduce win large ones at every M from 2^18 to 2^33, Zipf or uniform ids.
-// Measured on GB300 (ms per step, atomic against sorted):
-//   L = 32, Criteo-TB shape:     3.4M adds 0.045 / 0.055, 6.8M adds 0.074 / 0.059
-//   L = 16, Criteo-Kaggle shape: 6.8M adds 0.087 / 0.118, 13.6M adds 0.186 / 0.138
-// (blocks shorter than a warp leave the sorted reduce's lanes partly idle, so
-// its crossover lies higher).
+// Measured on GB300 (us of a whole step, atomic against sorted with the local
+// sort):
+//   L = 32, Criteo-TB shape, M = 2^18: 3.4M adds 38 / 27, 4.7M adds 40 / 29
+//   L = 16, Criteo-Kaggle shape, M = 2^20: 3.4M adds 52 / 42, 6.8M adds 94 / 49,
+//     13.6M adds 211 / 66
+//   L = 8, micro-benchmark shape, M = 2^18: 5.0M adds 71 / 43, 34M adds 261 / 157
+//   L = 64, 16.6M adds 127 / 62
+// (3.4M adds stay atomic as they were).  Without the local sort (run-to-run
+// identical bits, a forced global sort, shorter or untiled blocks) the sorted
+// path starts at 5M adds with blocks of 32 and more, 10M below; the fp32
+// atomic path is faster than the fp64 one and keeps those thresholds too.
 constexpr int64_t kSortedMaxR = int64_t(0xffffffffLL);
 
-int64_t auto_sorted_min_adds(int32_t L) { return L >= 32 ? 5000000 : 10000000; }
+int64_t auto_sorted_min_adds(const pss_handle* h) {
+    const DevParams& p = h->dp;
+    const bool local = h->sort_scope != PSS_SORT_GLOBAL && !h->deterministic &&
+                       h->accum == PSS_ACCUM_F64 &&
+                       ((p.Z == 32 && p.d % 32 == 0) ||
+                        (p.L >= 8 && local_reduce_ok(p) && (int64_t)p.R <= kCountSortMaxR));
+    return local ? 3500000 : p.L >= 32 ? 5000000 : 10000000;
+}
 
 bool sorted_supported(const pss_handle* h, int64_t nnz, int64_t B) {
     const int64_t J = h->dp.J;
@@ -419,7 +432,7 @@ bool use_radix(const pss_handle* h) {
 bool want_sorted(const pss_handle* h, int64_t npairs) {
     if (h->path == PSS_PATH_SORTED) return true;
     if (h->path == PSS_PATH_ATOMIC) return false;
-    return npairs * (int64_t)h->dp.L >= auto_sorted_min_adds(h->dp.L);
+    return npairs * (int64_t)h->dp.L >= auto_sorted_min_adds(h);
 }
 
 pss_status ensure_sorted(pss_handle* h, int64_t nnz, cudaStream_t st) {
@@ -855,8 +868,18 @@ constexpr int64_t kLocalMaxRereadPairsPerStart = 30;
 static LocalSort use_local_sort(const pss_handle* h, int64_t npairs, bool touch,
                                 const float* dgrad) {
     const int64_t R = (int64_t)h->dp.R;
-    if (h->deterministic || h->sort_scope == PSS_SORT_GLOBAL || !local_sort_ok(h->dp, dgrad))
-        return kLocalNo;
+    if (h->deterministic || h->sort_scope == PSS_SORT_GLOBAL) return kLocalNo;
+    if (!local_sort_ok(h->dp, dgrad)) {
+        // other chunk shapes: always counted, in batches that AUTO would sort
+        // (smaller ones leave the local sort's CTAs idle).  Measured on GB300,
+        // us of a whole step, global against local: micro-benchmark shape, M =
+        // 2^21, Z = 4, 8, 16, 64: 413 / 284, 230 / 154, 169 / 117, 122 / 110;
+        // Criteo-Kaggle shape, batch 32768: 136 / 66
+        return local_reduce_ok(h->dp) && !touch && R <= kCountSortMaxR &&
+                       npairs * (int64_t)h->dp.L >= auto_sorted_min_adds(h)
+                   ? kLocalCounted
+                   : kLocalNo;
+    }
     if (h->sort_scope == PSS_SORT_LOCAL || R > kCountSortMaxR ||
         npairs <= (int64_t)PSS_SORT_LOCAL_MAX_PAIRS_PER_START * R)
         return kLocalUncounted;

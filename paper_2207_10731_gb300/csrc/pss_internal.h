@@ -125,6 +125,8 @@ cudaError_t launch_mark_pairs(const SortedBuffers& sb, int64_t npairs, uint32_t 
 // staged reduce (local_sort_ok) with R < 2^32 - 1; any R, no per-bucket state.
 int64_t local_segments(int64_t npairs);
 bool local_sort_ok(const DevParams& p, const float* gout);
+// Other chunk shapes whose reduce takes the local layout.
+bool local_reduce_ok(const DevParams& p);
 // With `touched`, also the touched bitmap and list of the buckets.
 cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
                               const Touched* touched, int sm_count, cudaStream_t st);

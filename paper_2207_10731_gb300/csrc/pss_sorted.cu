@@ -981,6 +981,13 @@ k_range_reduce(const unsigned long long* __restrict__ sorted_e,
     if (count_runs && lg == 0 && nstart) atomicAdd(stats + 1, (unsigned long long)nstart);
 }
 
+// The buckets of 32 entries (one per lane, kBad for none) in which a run starts
+// are marked; the first entry's run may have started before.
+__device__ __forceinline__ void mark_heads(uint32_t x, uint8_t* __restrict__ seen, int lane) {
+    const uint32_t xp = __shfl_up_sync(0xffffffffu, x, 1);
+    if (seen && x != kBad && (lane == 0 || x != xp)) seen[x] = 1;
+}
+
 // Reduce for blocks of at least 32 elements: one WARP per task of kPiece
 // sorted entries, lane z owning elements z, z+32, ... of the block, so every
 // branch is warp-uniform and a run's sum goes straight from the lanes to the
@@ -994,15 +1001,19 @@ static_assert(kWU == 8, "the warp reduce sums kWU = 8 entries as a tree");
 // (at most 64 registers for KE <= 2: 4 CTAs per SM; at 72 registers, 3 per
 // SM, the paper micro-benchmark shape with Z = 64 reduced in 0.085 ms
 // against 0.073 ms with the bound)
-template <int KE, bool ZDIV, bool JPOW2>
+template <int KE, bool ZDIV, bool JPOW2, bool LOCAL>
 __global__ void __launch_bounds__(kThreads, (KE <= 2) ? 4 : 1)
 k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
                     unsigned long long* __restrict__ stats, int64_t npairs,
                     const float* __restrict__ gout, int d, int Z, int J, int log2J, int L,
-                    int64_t G, uint32_t smask, double* __restrict__ g, bool count_runs) {
+                    int64_t G, uint32_t smask, double* __restrict__ g, bool count_runs,
+                    const uint32_t* __restrict__ segn, uint8_t* __restrict__ seen) {
     pdl_prologue();
     __shared__ unsigned long long s_ent[kWarps][kPiece];
-    const int64_t total = (int64_t)(stats[0] < (unsigned long long)npairs ? stats[0] : npairs);
+    // (LOCAL: the segment-local layout, kLS / kPiece tasks per segment)
+    const int64_t total =
+        LOCAL ? ((npairs + kLS - 1) / kLS) * kLS
+              : (int64_t)(stats[0] < (unsigned long long)npairs ? stats[0] : npairs);
     const int64_t ntasks = (total + kPiece - 1) / kPiece;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -1022,15 +1033,24 @@ k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
     uint32_t nstart = 0;   // distinct buckets: entries whose bucket differs from the one before
     for (int64_t t = (int64_t)blockIdx.x * kWarps + warp; t < ntasks; t += wstride) {
         const int64_t e0 = t * kPiece;
-        const int n = (int)((e0 + kPiece < total) ? kPiece : total - e0);
+        int n = (int)((e0 + kPiece < total) ? kPiece : total - e0);
+        if (LOCAL) {
+            const int left = (int)__ldg(segn + (e0 >> kLSLog2)) - (int)(e0 & (kLS - 1));
+            if (left <= 0) continue;
+            if (left < n) n = left;
+        }
 #pragma unroll
-        for (int h = 0; h < (int)kPiece; h += 32)
-            ent[h + lane] = (h + lane < n) ? __ldg(sorted_e + e0 + h + lane) : kNone;
+        for (int h = 0; h < (int)kPiece; h += 32) {
+            const unsigned long long en =
+                (h + lane < n) ? __ldg(sorted_e + e0 + h + lane) : kNone;
+            ent[h + lane] = en;
+            if (LOCAL) mark_heads((uint32_t)(en >> 32), seen, lane);
+        }
         __syncwarp();
 #pragma unroll
         for (int k = 0; k < KE; ++k) s[k] = c[k] = 0.f;
         uint32_t cur = (uint32_t)(ent[0] >> 32);
-        if (count_runs)
+        if (!LOCAL && count_runs)
             nstart += (e0 == 0 || (uint32_t)(__ldg(sorted_e + e0 - 1) >> 32) != cur) ? 1u : 0u;
         for (int b = 0; b < n; b += kWU) {
             uint32_t xs[kWU];
@@ -1058,7 +1078,14 @@ k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
                     v[u][k] = (xs[u] != kBad && z < Lj) ? sign_by(__ldcs(src + z), sb) : 0.f;
                 }
             }
-            if (xs[kWU - 1] == cur) {
+            // (in bucket order the last entry tells; buckets that share a slot of
+            // the local sort interleave)
+            bool same = xs[kWU - 1] == cur;
+            if (LOCAL) {
+#pragma unroll
+                for (int u = 0; u < kWU - 1; ++u) same &= xs[u] == cur;
+            }
+            if (same) {
 #pragma unroll
                 for (int k = 0; k < KE; ++k) {
                     const float a = (v[0][k] + v[1][k]) + (v[2][k] + v[3][k]);
@@ -1082,7 +1109,79 @@ k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
         flush(cur);
         __syncwarp();
     }
-    if (count_runs && lane == 0 && nstart) atomicAdd(stats + 1, (unsigned long long)nstart);
+    if (!LOCAL && count_runs && lane == 0 && nstart) atomicAdd(stats + 1, (unsigned long long)nstart);
+}
+
+// Reduce of a local sort's short chunks (L = 4, 8 or 16 elements that tile the
+// rows): groups of L lanes, lane z of a group on element z, each group summing
+// kGS consecutive entries of its own (compensated) and adding every run's sum
+// once into the fp64 accumulator.  A warp stages the entries of its 32 / L
+// groups in shared memory with coalesced loads, and a group has 8 chunks in
+// flight.  What bounds it: instruction issue, about 25 per step of 32 / L
+// entries.  The entries of a segment read one piece of the gradient, so the
+// sectors of a line that other groups read come from L2.  Measured on GB300 at
+// the micro-benchmark shape with Z = 8: 74 us with a local sort of 25 us,
+// against 97 and 88 us for k_range_reduce after the global sort, whose random
+// 32-byte reads fetched the gradient three times.
+constexpr int kGS = 64;   // entries per group
+constexpr int kGU = 8;    // chunks in flight per group
+
+template <int LOG2L, bool SG>
+__global__ void __launch_bounds__(kThreads)
+k_group_reduce(const unsigned long long* __restrict__ sorted_e, int64_t npairs,
+               const uint32_t* __restrict__ segn, const float* __restrict__ gout, uint32_t G,
+               double* __restrict__ g, uint8_t* __restrict__ seen) {
+    pdl_prologue();
+    constexpr int E = 32 >> LOG2L;            // groups per warp
+    constexpr int kPer = E * kGS;             // entries per warp
+    static_assert(kLS % kPer == 0, "a warp's entries lie in one segment");
+    // (groups kGS + 1 entries apart, so that they read different banks)
+    __shared__ unsigned long long s_ent[kWarps][kPer + E];
+    const int lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
+    const int64_t e0 = ((int64_t)blockIdx.x * kWarps + warp) * kPer;
+    if (e0 >= npairs) return;
+    const int left = (int)__ldg(segn + (e0 >> kLSLog2)) - (int)(e0 & (kLS - 1));
+    if (left <= 0) return;
+    const int n = left < kPer ? left : kPer;
+    constexpr unsigned long long kNone = (unsigned long long)kBad << 32;
+#pragma unroll
+    for (int h = 0; h < kPer; h += 32) {
+        const unsigned long long en = h + lane < n ? __ldcs(sorted_e + e0 + h + lane) : kNone;
+        s_ent[warp][h + lane + (h + lane) / kGS] = en;
+        mark_heads((uint32_t)(en >> 32), seen, lane);
+    }
+    __syncwarp();
+    const int grp = lane >> LOG2L, z = lane & ((1 << LOG2L) - 1);
+    const unsigned long long* ent = &s_ent[warp][grp * (kGS + 1)];
+    const float* gz = gout + z;
+    double* const gl = g + z;
+    uint32_t cur = (uint32_t)(ent[0] >> 32);
+    float sum = 0.f, comp = 0.f;
+    const int steps = n < kGS ? n : kGS;      // of the first group, the longest
+    for (int i0 = 0; i0 < steps; i0 += kGU) {
+        uint32_t x[kGU];
+        float v[kGU];
+#pragma unroll
+        for (int u = 0; u < kGU; ++u) {
+            // (past the valid entries: chunk 0 is read and never added)
+            const unsigned long long en = ent[i0 + u];
+            x[u] = (uint32_t)(en >> 32);
+            const uint32_t r = SG ? (uint32_t)en & 0x7fffffffu : (uint32_t)en;
+            v[u] = __ldg(gz + ((uint64_t)r << LOG2L));
+            if (SG) v[u] = sign_by(v[u], (uint32_t)en & 0x80000000u);
+        }
+#pragma unroll
+        for (int u = 0; u < kGU; ++u) {
+            if (x[u] != cur) {
+                if (cur != kBad) red_add_f64(gl + (uint64_t)cur * G, widen(sum));
+                cur = x[u];
+                sum = comp = 0.f;
+            }
+            kahan_add(sum, comp, v[u]);
+        }
+    }
+    if (cur != kBad) red_add_f64(gl + (uint64_t)cur * G, widen(sum));
 }
 
 // Reduce for 32-element chunks that tile the rows (Z = 32 dividing d).  Each
@@ -1437,29 +1536,43 @@ k_window_combine(const unsigned long long* __restrict__ sorted_e,
 
 template <int KE, bool ZDIV, bool JPOW2>
 cudaError_t warp_reduce_launch(const SortedBuffers& sb, int64_t npairs, const float* gout,
-                               const DevParams& p, double* g, int log2J, bool count_runs,
-                               int sm_count, cudaStream_t st) {
+                               const DevParams& p, double* g, int log2J, bool local,
+                               bool count_runs, uint8_t* seen, int sm_count, cudaStream_t st) {
     const int64_t ntasks = (npairs + kPiece - 1) / kPiece;   // upper bound
-    const int grid = grid_for(k_warp_range_reduce<KE, ZDIV, JPOW2>, sm_count,
-                              (ntasks + kWarps - 1) / kWarps);
-    return launch_k(k_warp_range_reduce<KE, ZDIV, JPOW2>, dim3(grid), dim3(kThreads), 0, st,
-                    sb.sorted_e, sb.stats, npairs, gout, p.d, p.Z, p.J, log2J, p.L, p.G, p.smask, g,
-                    count_runs);
+    const auto kern = local ? k_warp_range_reduce<KE, ZDIV, JPOW2, true>
+                            : k_warp_range_reduce<KE, ZDIV, JPOW2, false>;
+    const int grid = grid_for(kern, sm_count, (ntasks + kWarps - 1) / kWarps);
+    return launch_k(kern, dim3(grid), dim3(kThreads), 0, st, sb.sorted_e, sb.stats, npairs, gout,
+                    p.d, p.Z, p.J, log2J, p.L, p.G, p.smask, g, count_runs, sb.segn, seen);
 }
 
 template <int KE>
 cudaError_t warp_reduce_inst(const SortedBuffers& sb, int64_t npairs, const float* gout,
-                             const DevParams& p, double* g, bool count_runs, int sm_count,
-                             cudaStream_t st) {
+                             const DevParams& p, double* g, bool local, bool count_runs,
+                             uint8_t* seen, int sm_count, cudaStream_t st) {
     const int log2J = (p.J & (p.J - 1)) == 0 ? ceil_log2(p.J) : -1;
     if (p.d % p.Z == 0)
-        return warp_reduce_launch<KE, true, true>(sb, npairs, gout, p, g, 0, count_runs, sm_count,
-                                                  st);
+        return warp_reduce_launch<KE, true, true>(sb, npairs, gout, p, g, 0, local, count_runs,
+                                                  seen, sm_count, st);
     if (log2J >= 0)
-        return warp_reduce_launch<KE, false, true>(sb, npairs, gout, p, g, log2J, count_runs,
-                                                   sm_count, st);
-    return warp_reduce_launch<KE, false, false>(sb, npairs, gout, p, g, 0, count_runs, sm_count,
-                                                st);
+        return warp_reduce_launch<KE, false, true>(sb, npairs, gout, p, g, log2J, local, count_runs,
+                                                   seen, sm_count, st);
+    return warp_reduce_launch<KE, false, false>(sb, npairs, gout, p, g, 0, local, count_runs, seen,
+                                                sm_count, st);
+}
+
+template <int LOG2L>
+cudaError_t group_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
+                         const DevParams& p, double* g, uint8_t* seen, cudaStream_t st) {
+    const auto kern = p.smask ? k_group_reduce<LOG2L, true> : k_group_reduce<LOG2L, false>;
+    const int64_t per = (int64_t)(32 >> LOG2L) * kGS * kWarps;   // entries per CTA
+    return launch_k(kern, dim3((unsigned)((npairs + per - 1) / per)), dim3(kThreads), 0, st,
+                    sb.sorted_e, npairs, sb.segn, gout, (uint32_t)p.G, g, seen);
+}
+
+// Chunks that tile the rows (chunk r starts at r*L) of 4, 8 or 16 elements.
+bool group_reduce_ok(const DevParams& p) {
+    return (p.L == 4 || p.L == 8 || p.L == 16) && (p.J == 1 || p.d % p.Z == 0);
 }
 
 template <int VW, int KC, bool JPOW2, bool ZDIV>
@@ -1669,6 +1782,10 @@ int64_t local_segments(int64_t npairs) { return (npairs + kLS - 1) / kLS; }
 
 bool local_sort_ok(const DevParams& p, const float* gout) { return window_reduce_ok(p, gout); }
 
+bool local_reduce_ok(const DevParams& p) {
+    return group_reduce_ok(p) || (p.L >= 32 && p.L <= 128);
+}
+
 cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
                               const Touched* touched, int sm_count, cudaStream_t st) {
     if (npairs <= 0) return cudaSuccess;
@@ -1698,7 +1815,7 @@ cudaError_t launch_count_seen(const SortedBuffers& sb, int64_t npairs, int64_t R
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
                                  bool reread, uint8_t* seen, int sm_count, cudaStream_t st) {
-    if (local && !window_reduce_ok(p, gout)) return cudaErrorInvalidValue;
+    if (local && !window_reduce_ok(p, gout) && !local_reduce_ok(p)) return cudaErrorInvalidValue;
     // 32-element chunks tiling the rows: asynchronous shared-memory staging
     if (window_reduce_ok(p, gout)) {
         if (local)
@@ -1711,10 +1828,17 @@ cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const 
     }
     // blocks of 32+ elements: one warp per task, one element per lane
     if (p.L >= 32) {
-        if (p.L <= 32) return warp_reduce_inst<1>(sb, npairs, gout, p, g, count_runs, sm_count, st);
-        if (p.L <= 64) return warp_reduce_inst<2>(sb, npairs, gout, p, g, count_runs, sm_count, st);
-        if (p.L <= 128)
-            return warp_reduce_inst<4>(sb, npairs, gout, p, g, count_runs, sm_count, st);
+#define PSS_WR(KE) \
+    return warp_reduce_inst<KE>(sb, npairs, gout, p, g, local, count_runs, seen, sm_count, st)
+        if (p.L <= 32) PSS_WR(1);
+        if (p.L <= 64) PSS_WR(2);
+        if (p.L <= 128) PSS_WR(4);
+#undef PSS_WR
+    }
+    if (local) {
+        if (p.L == 4) return group_reduce<2>(sb, npairs, gout, p, g, seen, st);
+        if (p.L == 8) return group_reduce<3>(sb, npairs, gout, p, g, seen, st);
+        return group_reduce<4>(sb, npairs, gout, p, g, seen, st);
     }
     const bool vec = (p.Z % 4 == 0) && (p.d % 4 == 0) && (((uintptr_t)gout & 15u) == 0);
     const int vw = vec ? 4 : 1;

@@ -82,3 +82,40 @@ def test_local_sort_touched_list(B):
         h.close()
     np.testing.assert_array_equal(state[0][0], state[1][0])
     np.testing.assert_array_equal(state[0][1], state[1][1])
+
+
+@pytest.mark.parametrize("signed", [False, True], ids=["unsigned", "signed"])
+@pytest.mark.parametrize("d,Z,B", [(32, 8, 20001), (64, 4, 9000), (16, 32, 45000), (128, 64, 6007),
+                                   (96, 64, 5200), (50, 8, 15000), (256, 128, 2800),
+                                   (32, 8, 30011), (64, 4, 11003)])
+def test_local_reduce_of_other_chunks_bit_exact(d, Z, B, signed):
+    # chunks of other lengths, in batches large enough for the local sort
+    # (its buckets that share a slot interleave), and rows that they do not tile
+    w = wl.make_workload("tiny", T=15, d=d, Z=Z, M=9000, B=B, cards=("const", 900), bag=("one",),
+                         ids=("zipf", 1.05), grad="dyadic", w0="dyadic")
+    idx = w.indices.copy()
+    idx[4::13] = 900                                   # dropped
+    h = binding.PSS(w.cards, dim=w.d, M=w.M, Z=w.Z, G=w.G, seed=w.seed, optimizer="sgd")
+    o = oracle.OraclePSS(w.cards, d=w.d, M=w.M, Z=w.Z, G=w.G, seed=w.seed, signed=signed)
+    h.set_option(binding.OPT_SIGNED, int(signed))
+    h.set_weights(gu.cuda(w.w0))
+    locs, _ = o.locations(idx, w.offsets, B)
+    locs = locs[locs >= 0]
+    h.forward(gu.cuda(idx), gu.cuda(w.offsets), B)
+    got = gu.host(h.backward_grad(gu.cuda(w.grad_out)))
+    want = o.grad(idx, w.offsets, B, w.grad_out)
+    # k / 2^8 with |k| < 2^10, summed over at most 2^20 terms: exact in fp64
+    # and in every partial sum below 2^16, beyond which fp32 may round once
+    small = np.abs(want) < 2.0 ** 15
+    np.testing.assert_array_equal(got[small], want.astype(np.float32)[small])
+    np.testing.assert_allclose(got, want, rtol=2.0 ** -20, atol=0)
+    gu.torch().cuda.synchronize()
+    # AUTO sorts batches that add 3.5M elements with blocks that the local sort
+    # serves, 10M with blocks of 4; smaller ones take the atomic path, which
+    # counts nothing
+    if w.nnz * h.J * h.L < (3_500_000 if h.L >= 8 else 10_000_000):
+        assert h.info()["last_path"] == binding.PATH_ATOMIC
+    else:
+        assert h.info()["last_path"] == binding.PATH_SORTED
+        assert h.info()["last_collision_rate"] == 1.0 - np.unique(locs).shape[0] / locs.shape[0]
+    h.close()
