@@ -157,6 +157,16 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Device memory of device `dev` itself.
+bool is_own_device_ptr(const void* p, int dev) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == dev;
+}
+
 cudaError_t ensure(Staging& s, size_t bytes, cudaStream_t st) {
     if (bytes == 0) bytes = 16;
     if (s.cap >= bytes) return cudaSuccess;
@@ -253,6 +263,19 @@ pss_status grad_release(pss_handle* h, bool staged, cudaStream_t st) {
         h->grad_free_pending = true;
     }
     return PSS_OK;
+}
+
+// The array (n == M values from the library's buffer `src`) to the caller.  A
+// kernel where both lie in this device's memory and fit in L2: it is launched
+// behind the kernel before it without a gap, and reads what the update left in
+// L2.  Measured on GB300 for 2.5M values: 3.6 us against 7.5 for the runtime's
+// copy, and 6 us less for a whole Criteo-TB step of 2048 rows.  Larger arrays
+// move at HBM rate either way (2^26 values: 82 us).
+constexpr int64_t kCopyKernelMax = int64_t(1) << 24;
+pss_status copy_out(pss_handle* h, float* dst, const float* src, int64_t n, cudaStream_t st) {
+    if (n <= kCopyKernelMax && ((uintptr_t)dst & 15u) == 0 && is_own_device_ptr(dst, h->device))
+        return cuda_status(launch_copy(src, dst, n, h->sm_count, st));
+    return cuda_status(cudaMemcpyAsync(dst, src, sizeof(float) * (size_t)n, cudaMemcpyDefault, st));
 }
 
 EventPair take_events(pss_handle* h) {
@@ -697,19 +720,16 @@ pss_status pss_set_weights(pss_handle* h, const float* w, int64_t n, pss_stream 
 pss_status pss_get_weights(pss_handle* h, float* w, int64_t n, pss_stream stream) {
     if (!h || !w || n != h->dp.M) return PSS_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
-    PSS_TRY(cudaMemcpyAsync(w, h->w, sizeof(float) * (size_t)n, cudaMemcpyDefault,
-                            reinterpret_cast<cudaStream_t>(stream)));
-    return PSS_OK;
+    return copy_out(h, w, h->w, n, reinterpret_cast<cudaStream_t>(stream));
 }
 
 pss_status pss_get_state(pss_handle* h, float* w, float* G, int64_t n, pss_stream stream) {
     if (!h || !w || n != h->dp.M || (h->opt == PSS_ADAGRAD && !G)) return PSS_ERR_INVALID_ARG;
     DeviceGuard g(h->device);
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    PSS_TRY(cudaMemcpyAsync(w, h->w, sizeof(float) * (size_t)n, cudaMemcpyDefault, st));
-    if (h->opt == PSS_ADAGRAD)
-        PSS_TRY(cudaMemcpyAsync(G, h->Gacc, sizeof(float) * (size_t)n, cudaMemcpyDefault, st));
-    return PSS_OK;
+    const pss_status rc = copy_out(h, w, h->w, n, st);
+    if (rc != PSS_OK || h->opt != PSS_ADAGRAD) return rc;
+    return copy_out(h, G, h->Gacc, n, st);
 }
 
 pss_status pss_set_state(pss_handle* h, const float* w, const float* G, int64_t n,

@@ -195,6 +195,8 @@ cudaError_t launch_update_touched(bool adagrad, float* w, float* Gacc, float* g,
 cudaError_t launch_update_touched64(bool adagrad, float* w, float* Gacc, double* g,
                                     const Touched& touched, int64_t G, int32_t L, float lr,
                                     float eps, int sm_count, cudaStream_t st);
+// out[i] = in[i] for i < n (device memory, 16-byte aligned).
+cudaError_t launch_copy(const float* in, float* out, int64_t n, int sm_count, cudaStream_t st);
 // out[e] = fp32(g[e]); g[e] = 0 for all e < M.
 cudaError_t launch_grad_export(double* g, float* out, int64_t M, int sm_count, cudaStream_t st);
 // Clears the bitmap words of the listed starts and resets the list count.

@@ -156,6 +156,25 @@ k_convert(int direction, const void* __restrict__ in, void* __restrict__ out, in
     }
 }
 
+// out[0 .. n) = in, 16-byte aligned both.  What bounds it: L2 (the caller copies
+// arrays that fit there; the update has just written them).
+__global__ void __launch_bounds__(kThreads)
+k_copy(const float* __restrict__ in, float* __restrict__ out, int64_t n) {
+    pdl_prologue();
+    const int64_t n4 = n >> 2, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const float4* in4 = reinterpret_cast<const float4*>(in);
+    float4* out4 = reinterpret_cast<float4*>(out);
+    int64_t i = i0;
+    for (; i + stride < n4; i += 2 * stride) {
+        const float4 a = in4[i], b = in4[i + stride];
+        out4[i] = a;
+        out4[i + stride] = b;
+    }
+    if (i < n4) out4[i] = in4[i];
+    if (i0 < (n & 3)) out[n4 * 4 + i0] = in[n4 * 4 + i0];
+}
+
 // Gradient export: out[e] = fp32(g[e]) and g[e] = 0, over all of M.
 __global__ void __launch_bounds__(kThreads)
 k_grad_export(double* __restrict__ g, float* __restrict__ out, int64_t M) {
@@ -324,6 +343,11 @@ cudaError_t launch_update_touched64(bool adagrad, float* w, float* Ga, double* g
 cudaError_t launch_grad_export(double* g, float* out, int64_t M, int sm_count, cudaStream_t st) {
     const int grid = grid_for(k_grad_export, sm_count, (M + kThreads - 1) / kThreads);
     return launch_k(k_grad_export, dim3(grid), dim3(kThreads), 0, st, g, out, M);
+}
+
+cudaError_t launch_copy(const float* in, float* out, int64_t n, int sm_count, cudaStream_t st) {
+    const int grid = grid_for(k_copy, sm_count, ((n >> 2) + kThreads) / kThreads);
+    return launch_k(k_copy, dim3(grid), dim3(kThreads), 0, st, in, out, n);
 }
 
 cudaError_t launch_fold_tail(double* g64, float* g32, int64_t M, int L, cudaStream_t st) {
