@@ -297,11 +297,14 @@ __device__ __forceinline__ void emit_pairs(const XT* s_x, int n, int J, uint32_t
 
 // Bags of any length: pools the nb bags of a tile, lane l holding the offsets
 // [q0, q1) of bag l (mod the power of two at or above the tile's bags), all
-// ids within [qa, qb).  The ids are staged and hashed in windows; the whole
-// warp takes one bag at a time; its ng lane groups add ng consecutive ids of
-// the bag in parallel, kUM steps per round.  A round's kUM values are summed
+// ids within [qa, qb).  The ids are staged and hashed in windows.  Bags of
+// similar length that lie inside a window go one to a lane group, ng at a
+// time.  Other bags take the whole warp, one at a time: its ng lane groups add
+// ng consecutive ids of the bag in parallel, kUM steps per round.  A round's kUM values are summed
 // as a tree and added with compensation; at the end of the bag the groups'
 // sums are merged the same way and group 0 stores the row.
+// (One bag per lane group needs no merge and fewer partly filled rounds: 234
+// us per multi-hot forward against 244 with the whole warp on every bag.)
 // What bounds it: instruction issue, then the L2 gathers.  So whole rounds of
 // valid ids run without tests, the sums take two elements per instruction, an
 // id's chunks are hashed from one product, and a bag's bounds in the window
@@ -326,6 +329,7 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
     const int64_t qb = __shfl_sync(0xffffffffu, q1, nb - 1);
     int64_t sw0 = __shfl_sync(0xffffffffu, q0, 0);
     int bi = 0;
+    bool begun = false;              // bag bi has ids in an earlier window
     Sum<VW> acc[KC];
     for (;;) {
         // stage the window [sw0, sw0 + n)
@@ -354,7 +358,67 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
         const int64_t a = q0 - sw0, c = q1 - sw0;
         const int lo = (int)(a < 0 ? 0 : a < n ? a : n), hi = (int)(c < n ? c : n);
         const unsigned ends = __ballot_sync(0xffffffffu, c <= n);
-        for (; bi < nb; ++bi) {
+        while (bi < nb) {
+            if (ng > 1 && clean && bi + ng <= nb && ((ends >> (bi + ng - 1)) & 1u)) {
+                // ng bags that end in this window, the first not begun before
+                // it: one per lane group, unless one is much longer than the rest
+                const int b0 = __shfl_sync(0xffffffffu, lo, bi + g);
+                const int m = __shfl_sync(0xffffffffu, hi, bi + g) - b0;
+                int mx = m, mn = m, sum = m;
+                for (int o = gs; o < 32; o <<= 1) {
+                    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                    mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+                    sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                }
+                if (!begun && mx * ng <= 2 * sum + 8 * ng) {
+                    if (q_row)
+                        for (int i = lane & (gs - 1); i < m; i += gs)
+                            q_row[sw0 + b0 + i] = row + (uint32_t)g * (uint32_t)p.T;
+                    Sum<VW> ga[KC];
+                    const XT* sx = s_x + b0 * J;
+                    int left = mn;
+                    for (; left >= kUM; left -= kUM) {   // rounds that every bag fills
+                        VT v[kUM][KC];
+#pragma unroll
+                        for (int u = 0; u < kUM; ++u)
+#pragma unroll
+                            for (int k = 0; k < KC; ++k)
+                                v[u][k] = gather<SG, V>(wz[k], fg.Gb, sx[u * J + col.js[k]]);
+                        sx += kUM * J;
+#pragma unroll
+                        for (int k = 0; k < KC; ++k) ga[k].add4(v[0][k], v[1][k], v[2][k], v[3][k]);
+                    }
+                    // the rest: groups past their bag load the window's first id
+                    // and drop it
+                    const int done = mn - left;
+                    for (int i = done; i < mx; i += kUM) {
+                        VT v[kUM][KC];
+#pragma unroll
+                        for (int u = 0; u < kUM; ++u) {
+                            const bool in = i + u < m;
+                            const XT* su = in ? sx + u * J : s_x;
+#pragma unroll
+                            for (int k = 0; k < KC; ++k) {
+                                v[u][k] = gather<SG, V>(wz[k], fg.Gb, su[col.js[k]]);
+#pragma unroll
+                                for (int c = 0; c < VW; ++c)
+                                    V::set(v[u][k], c, in ? V::get(v[u][k], c) : 0.f);
+                            }
+                        }
+                        sx += kUM * J;
+#pragma unroll
+                        for (int k = 0; k < KC; ++k) ga[k].add4(v[0][k], v[1][k], v[2][k], v[3][k]);
+                    }
+                    float* og = orow + g * ostride;
+#pragma unroll
+                    for (int k = 0; k < KC; ++k)
+                        if (col.v[k]) V::stcs(og + col.e[k], ga[k].value());
+                    orow += ng * ostride;
+                    row += (uint32_t)(ng * p.T);
+                    bi += ng;
+                    continue;
+                }
+            }
             const int b0 = __shfl_sync(0xffffffffu, lo, bi), b1 = __shfl_sync(0xffffffffu, hi, bi);
             if (q_row)   // the bag's ids' output row, one store per lane
                 for (int i = b0 + lane; i < b1; i += 32) q_row[sw0 + i] = row;
@@ -409,7 +473,8 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
                     for (int k = 0; k < KC; ++k) acc[k].add4(v[0][k], v[1][k], v[2][k], v[3][k]);
                 }
             }
-            if (!((ends >> bi) & 1u)) break;   // it goes on in the next window
+            begun = !((ends >> bi) & 1u);
+            if (begun) break;   // it goes on in the next window
             for (int o = gs; o < 32; o <<= 1)
 #pragma unroll
                 for (int k = 0; k < KC; ++k) acc[k].merge(o);
@@ -422,6 +487,7 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
             row += (uint32_t)p.T;
 #pragma unroll
             for (int k = 0; k < KC; ++k) acc[k] = Sum<VW>();
+            ++bi;
         }
         if (bi >= nb) break;
         sw0 += n;
