@@ -1333,10 +1333,16 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
         tb_start = (e1 < total) ? (int64_t)(uint32_t)(__ldg(sorted_e + e1) >> 32) * G : INT64_MAX;
         wb = hx;
     }
+    // (per run: the shift in 32 bits and one uniform test for the boundaries;
+    // with 64-bit positions compared per element 78 us per reduce against 73,
+    // batch 20011)
+    uint32_t wx = cur;                       // the window's bucket: wb = wx * G
     auto finalize = [&](int lim) {   // the window's first lim elements are done
-        if (lane < lim) {
+        const float v = acc - accc;
+        if (wb >= hb_end && wb + 32 <= tb_start) {   // inside the range (warp-uniform)
+            if (lane < lim && v != 0.f) ws.gexp[wb + lane] = v;
+        } else if (lane < lim) {
             const int64_t e = wb + lane;
-            const float v = acc - accc;
             if (e < hb_end || e >= tb_start) {
                 float* rec = ws.bnd + task * 64;
                 if (e < hx + 32) rec[e - hx] = v;
@@ -1352,20 +1358,18 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
             if (SINK == kSinkF64) {
                 red_add_f64(glane + (uint64_t)cur * G, widen(sum));
             } else {
-                const int64_t xb = (int64_t)cur * G;
-                const int64_t sh = xb - wb;           // >= 0: buckets ascend
-                if (sh > 0) {
-                    finalize(sh < 32 ? (int)sh : 32);
-                    if (sh >= 32) {
-                        acc = accc = 0.f;
-                    } else {
-                        const float a2 = __shfl_down_sync(0xffffffffu, acc, (int)sh);
-                        const float c2 = __shfl_down_sync(0xffffffffu, accc, (int)sh);
-                        const bool in = lane + (int)sh < 32;
-                        acc = in ? a2 : 0.f;
-                        accc = in ? c2 : 0.f;
-                    }
-                    wb = xb;
+                const uint32_t dx = cur - wx;         // buckets ascend
+                if (dx != 0u) {
+                    // (32 buckets on are past the window whatever G is)
+                    const uint32_t sh = dx >= 32u ? 32u : min(dx * (G < 32u ? G : 32u), 32u);
+                    finalize((int)sh);
+                    const float a2 = __shfl_down_sync(0xffffffffu, acc, sh & 31u);
+                    const float c2 = __shfl_down_sync(0xffffffffu, accc, sh & 31u);
+                    const bool in = lane + (int)sh < 32;
+                    acc = in ? a2 : 0.f;
+                    accc = in ? c2 : 0.f;
+                    wx = cur;
+                    wb = (int64_t)cur * G;
                 }
                 kahan_add(acc, accc, sum - comp);
             }
