@@ -303,13 +303,15 @@ __device__ __forceinline__ void emit_pairs(const XT* s_x, int n, int J, uint32_t
 // ng consecutive ids of the bag in parallel, kUM steps per round.  A round's kUM values are summed
 // as a tree and added with compensation; at the end of the bag the groups'
 // sums are merged the same way and group 0 stores the row.
-// (One bag per lane group needs no merge and fewer partly filled rounds: 234
-// us per multi-hot forward against 244 with the whole warp on every bag.)
+// (One bag per lane group, GROUPS, needs no merge and fewer partly filled
+// rounds: 234 us per multi-hot forward against 244 with the whole warp on
+// every bag.  The variants for one-id bags leave it out: its registers cost
+// them 10-40%.)
 // What bounds it: instruction issue, then the L2 gathers.  So whole rounds of
 // valid ids run without tests, the sums take two elements per instruction, an
 // id's chunks are hashed from one product, and a bag's bounds in the window
 // are 32-bit numbers that the lanes compute together.
-template <int VW, int KC, typename XT, bool SG>
+template <int VW, int KC, typename XT, bool SG, bool GROUPS>
 __device__ __forceinline__ void
 forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ idx, uint32_t tJ,
              uint64_t card, int64_t q0, int64_t q1, int nb, XT* s_x,
@@ -359,7 +361,7 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
         const int lo = (int)(a < 0 ? 0 : a < n ? a : n), hi = (int)(c < n ? c : n);
         const unsigned ends = __ballot_sync(0xffffffffu, c <= n);
         while (bi < nb) {
-            if (ng > 1 && clean && bi + ng <= nb && ((ends >> (bi + ng - 1)) & 1u)) {
+            if (GROUPS && ng > 1 && clean && bi + ng <= nb && ((ends >> (bi + ng - 1)) & 1u)) {
                 // ng bags that end in this window, the first not begun before
                 // it: one per lane group, unless one is much longer than the rest
                 const int b0 = __shfl_sync(0xffffffffu, lo, bi + g);
@@ -603,8 +605,9 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
                         V::stcs(obase + bi * ostride + col.e[k], z);
                     }
             } else {
-                forward_bags<VW, KC, XT, SG>(p, fg, idx, tJ, card, q0, q1, nb, s_x, wz, col, obase,
-                                             ostride, row0, err, pair_x, q_row, log2gs, lane);
+                forward_bags<VW, KC, XT, SG, MODE == kFwdLong>(
+                    p, fg, idx, tJ, card, q0, q1, nb, s_x, wz, col, obase, ostride, row0, err,
+                    pair_x, q_row, log2gs, lane);
             }
         } else {
             // every bag holds at most one id: s_x[bag*J + j] is the bucket of
