@@ -119,10 +119,11 @@ inline int ceil_log2(int v) {
     return l;
 }
 
-// CTAs of `threads` threads and `smem` bytes of dynamic shared memory (allowed
-// here where it is above the default 48 KB) that fit on an SM at once.  The
-// answer is a constant of the kernel and the device, and asking the runtime
-// costs about as much as a launch: each thread keeps what it was told.
+// CTAs of `threads` threads and `smem` bytes of dynamic shared memory that fit
+// on an SM at once; shared memory above the default 48 KB is allowed first (on
+// every call: it belongs to the context).  The answer is a constant of the
+// kernel and the device, and asking the runtime costs about as much as a
+// launch: each thread keeps what it was told.
 inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, int* per_sm) {
     struct Known {
         const void* kernel;
@@ -131,16 +132,17 @@ inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, i
     };
     constexpr int kKnown = 64;
     static thread_local Known known[kKnown] = {};
+    if (smem > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
     int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    const cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const size_t h = ((size_t)kernel >> 4) * 0x9e3779b97f4a7c15ull + smem;
     Known& k = known[(h >> 32) % kKnown];
     if (k.kernel != kernel || k.smem != smem || k.dev != dev || k.threads != threads) {
-        if (smem > 48 * 1024) {
-            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
         int n = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) !=
                 cudaSuccess ||

@@ -263,7 +263,7 @@ struct FwdGeom {
 // Buckets of chunks j0, j0 + lpi, ... of one id into sx[0 .. J), Invalid for a
 // bad id: one product A*key per lane, chunk j + lpi has step = A*lpi more.
 template <typename XT, bool SG>
-__device__ __forceinline__ void hash_id(const DevParams& p, uint64_t TJ, uint64_t id, uint32_t tJ,
+__device__ __forceinline__ void hash_id(const DevParams& p, uint64_t TJ, uint64_t id, uint64_t tJ,
                                         bool valid, int j0, int lpi, uint64_t step, uint64_t step2,
                                         XT* sx) {
     const uint64_t key = id * TJ + tJ + (uint32_t)j0;   // hash_key; tJ = t*J
@@ -313,7 +313,7 @@ __device__ __forceinline__ void emit_pairs(const XT* s_x, int n, int J, uint32_t
 // are 32-bit numbers that the lanes compute together.
 template <int VW, int KC, typename XT, bool SG, bool GROUPS>
 __device__ __forceinline__ void
-forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ idx, uint32_t tJ,
+forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ idx, uint64_t tJ,
              uint64_t card, int64_t q0, int64_t q1, int nb, XT* s_x,
              const float* const (&wz)[KC], const Cols<VW, KC>& col, float* orow, int64_t ostride,
              uint32_t row, DevError* err, uint32_t* __restrict__ pair_x,
@@ -587,7 +587,7 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
         const int nb = (int)((b_hi - b0) < wb ? (b_hi - b0) : wb);
         float* obase = out + b0 * ostride + (int64_t)t * p.d;
         const uint32_t row0 = (uint32_t)b0 * (uint32_t)p.T + (uint32_t)t;
-        const uint32_t tJ = (uint32_t)t * (uint32_t)J;
+        const uint64_t tJ = (uint64_t)(uint32_t)t * (uint32_t)J;
         const uint64_t card = (uint64_t)__ldg(p.cards + t);
         const bool has = q1 > q0;
         const unsigned odd = __ballot_sync(0xffffffffu, q0 < 0 || q1 < q0 || q1 > nnz);
