@@ -528,7 +528,7 @@ pss_status ensure_radix(pss_handle* h, int64_t npairs, cudaStream_t st) {
         h->radix_pairs_cap = 0;
         const size_t n = (size_t)(npairs > 0 ? npairs : 1);
         PSS_TRY(cudaMallocAsync(&h->sb.tmp_e, sizeof(unsigned long long) * n, st));
-        const size_t nc = (size_t)radix_tiles((int64_t)n) * (size_t)(1 << kRadixMaxBits);
+        const size_t nc = (size_t)radix_tiles((int64_t)n, h->sm_count) * (size_t)(1 << kRadixMaxBits);
         PSS_TRY(cudaMallocAsync(&h->sb.cnt, sizeof(uint32_t) * nc, st));
         h->radix_pairs_cap = npairs;
     }
@@ -940,7 +940,7 @@ static pss_status sort_pairs(pss_handle* h, bool touch, LocalSort local, cudaStr
         if (rc0 != PSS_OK) return rc0;
         const RadixPlan plan = radix_plan(h->dp.R, (int)h->sort_digit_bits);
         LaunchScope ls(h, PSS_K_SORT, st, 3 * plan.passes + (touch ? 1 : 0));
-        PSS_TRY(launch_radix_sort(h->sb, npairs, h->dp.J, h->dp.smask, plan, st));
+        PSS_TRY(launch_radix_sort(h->sb, npairs, h->dp.J, h->dp.smask, plan, h->sm_count, st));
         if (touch)
             PSS_TRY(launch_mark_pairs(h->sb, npairs, h->dp.smask, h->touched, h->sm_count, st));
     } else {

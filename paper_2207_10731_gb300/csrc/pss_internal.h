@@ -76,7 +76,7 @@ struct RadixPlan {
 // Plan for buckets in [0, R): digit_bits 0 picks at most kRadixMaxBits bits per
 // pass, as few passes as that allows, split evenly; 4 .. 11 forces that many.
 RadixPlan radix_plan(uint64_t R, int digit_bits);
-int64_t radix_tiles(int64_t npairs);   // tiles of one pass
+int64_t radix_tiles(int64_t npairs, int sm_count);   // tiles of a pass of up to npairs pairs, at most
 
 // Buffers of the sorted backward path (see pss_sorted.cu).
 struct SortedBuffers {
@@ -94,7 +94,7 @@ struct SortedBuffers {
     uint32_t* bnz;                // per scan chunk: non-empty buckets
     // radix sort
     unsigned long long* tmp_e;    // nnz*J entries: the other buffer of the radix passes
-    uint32_t* cnt;                // [2^bits][radix_tiles(nnz*J)] per-tile digit counts
+    uint32_t* cnt;                // [2^bits][tiles] per-tile digit counts
     uint32_t* tot;                // [2^kRadixMaxBits] digit totals of the current pass
     uint32_t* dstart;             // [2^kRadixMaxBits] digit start positions of the current pass
     uint32_t* done;               // finished-CTA counter of the column scan (zero between passes)
@@ -115,7 +115,7 @@ cudaError_t launch_sorted_scatter(const SortedBuffers& sb, int64_t npairs, int J
 // Stable radix sort of the forward's pairs by bucket into sorted_e (three
 // kernels per pass; see pss_sorted.cu): entries of one bucket in pair order.
 cudaError_t launch_radix_sort(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
-                              const RadixPlan& plan, cudaStream_t st);
+                              const RadixPlan& plan, int sm_count, cudaStream_t st);
 // Touched bitmap / list of the buckets of the forward's pairs.
 cudaError_t launch_mark_pairs(const SortedBuffers& sb, int64_t npairs, uint32_t smask,
                               const Touched& touched, int sm_count, cudaStream_t st);

@@ -467,8 +467,8 @@ k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
 // Stable LSD radix sort of the pairs by bucket x.
 //
 // The keys are the bucket indices (at most 32 bits); the sort makes P passes of
-// D <= 11 bits each (RadixPlan).  A pass cuts its input into TILES of kRTile
-// consecutive entries and takes three kernels:
+// D <= 11 bits each (RadixPlan).  A pass cuts its input into TILES of 256 * per
+// consecutive entries (per <= kRPer, see radix_per) and takes three kernels:
 //   up       each tile's count of every digit, cnt[digit][tile];
 //   colscan  for every digit, the exclusive prefix of its counts over the
 //            tiles (in place, one warp per digit) and its total; the last CTA
@@ -486,9 +486,10 @@ k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
 // valid pairs to stats[0], which the later passes and the reduce read.
 constexpr int kRThreads = 256;
 constexpr int kRWarps = kRThreads / 32;
-constexpr int kRPer = 32;                        // entries per thread and tile
-constexpr int kRWarpKeys = 32 * kRPer;           // entries per warp and tile
-constexpr int kRTile = kRThreads * kRPer;        // entries per tile
+constexpr int kRPer = 32;                        // entries per thread and tile at most
+constexpr int kRMinPer = 8;
+constexpr int kRWarpKeys = 32 * kRPer;           // entries per warp and tile at most
+constexpr int kRTile = kRThreads * kRPer;        // entries per tile at most
 constexpr int kRMaxDigits = 1 << kRadixMaxBits;
 constexpr int kRMaxOwn = kRMaxDigits / kRThreads; // digits per thread at most
 static_assert(kRWarpKeys < 65536, "per-warp digit counts are 16-bit");
@@ -544,22 +545,26 @@ __device__ __forceinline__ int64_t radix_count(int64_t npairs,
 
 // up: cnt[d][tile] = entries of the tile with digit d (every tile writes all
 // of its nd counts, zeros included).
-template <bool FIRST, bool SG>
+template <bool FIRST, bool SG, bool FULL>
 __global__ void __launch_bounds__(kRThreads)
 k_radix_up(const uint32_t* __restrict__ pair_x, const unsigned long long* __restrict__ in_e,
            int64_t npairs, const unsigned long long* __restrict__ stats, int shift, int bits,
-           int ntiles, uint32_t* __restrict__ cnt) {
+           int ntiles, int per_arg, uint32_t* __restrict__ cnt) {
     pdl_prologue();
+    const int per = FULL ? kRPer : per_arg;
     __shared__ uint32_t s_c[kRMaxDigits];
     const int nd = 1 << bits;
     const uint32_t dmask = (uint32_t)nd - 1u;
     for (int d = threadIdx.x; d < nd; d += kRThreads) s_c[d] = 0u;
     __syncthreads();
     const int64_t n = radix_count<FIRST>(npairs, stats);
-    const int64_t t0 = (int64_t)blockIdx.x * kRTile;
+    const int64_t t0 = (int64_t)blockIdx.x * (kRThreads * per);
     uint32_t hi[kRPer];
 #pragma unroll
+    for (int i = 0; i < kRPer; ++i) hi[i] = kBad;
+#pragma unroll
     for (int i = 0; i < kRPer; ++i) {
+        if (i >= per) break;
         const int64_t p = t0 + (int64_t)i * kRThreads + threadIdx.x;
         if (FIRST) {
             hi[i] = (p < n) ? __ldg(pair_x + p) : kBad;
@@ -660,14 +665,15 @@ __host__ __device__ constexpr size_t radix_down_smem(int nd) {
 }
 
 // down: one tile per CTA (see the section comment).
-template <bool FIRST, bool SG>
+template <bool FIRST, bool SG, bool FULL>
 __global__ void __launch_bounds__(kRThreads, 2)
 k_radix_down(const uint32_t* __restrict__ pair_x, const uint32_t* __restrict__ q_row,
              const unsigned long long* __restrict__ in_e, unsigned long long* __restrict__ out_e,
              int64_t npairs, const unsigned long long* __restrict__ stats, int J, int log2J,
-             int shift, int bits, int ntiles, const uint32_t* __restrict__ cnt,
+             int shift, int bits, int ntiles, int per_arg, const uint32_t* __restrict__ cnt,
              const uint32_t* __restrict__ dstart) {
     pdl_prologue();
+    const int per = FULL ? kRPer : per_arg;
     extern __shared__ __align__(16) unsigned char r_smem[];
     const int nd = 1 << bits;
     unsigned long long* s_tile = reinterpret_cast<unsigned long long*>(r_smem);   // [kRTile]
@@ -679,36 +685,43 @@ k_radix_down(const uint32_t* __restrict__ pair_x, const uint32_t* __restrict__ q
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int64_t n = radix_count<FIRST>(npairs, stats);
-    const int64_t t0 = (int64_t)blockIdx.x * kRTile;
+    const int64_t t0 = (int64_t)blockIdx.x * (kRThreads * per);
     if (t0 >= n) return;
     {
         uint32_t* z = reinterpret_cast<uint32_t*>(s_hist);
         for (int i = threadIdx.x; i < kRWarps * nd / 2; i += kRThreads) z[i] = 0u;
     }
-    // load, warp w taking entries t0 + w*kRWarpKeys + i*32 + lane (i in order)
+    // load, warp w taking entries t0 + w*32*per + i*32 + lane (i in order)
     unsigned long long e[kRPer];
+#pragma unroll
+    for (int i = 0; i < kRPer; ++i) e[i] = ~0ull;
     {
-        const int64_t wb = t0 + (int64_t)warp * kRWarpKeys + lane;
+        const int64_t wb = t0 + (int64_t)warp * (32 * per) + lane;
         if (FIRST) {
             // every load is issued before any is used: buckets, then id rows
             uint32_t x[kRPer], row[kRPer];
 #pragma unroll
             for (int i = 0; i < kRPer; ++i) {
+                if (i >= per) break;
                 const int64_t p = wb + i * 32;
                 x[i] = (p < n) ? __ldg(pair_x + p) : kBad;
             }
 #pragma unroll
             for (int i = 0; i < kRPer; ++i) {
+                if (i >= per) break;
                 const uint32_t pp = (uint32_t)(wb + i * 32);   // npairs < 2^32 here
                 const uint32_t q = (log2J >= 0) ? (pp >> log2J) : pp / (uint32_t)J;
                 row[i] = (wb + i * 32 < n) ? __ldg(q_row + q) : 0u;
             }
 #pragma unroll
-            for (int i = 0; i < kRPer; ++i)
+            for (int i = 0; i < kRPer; ++i) {
+                if (i >= per) break;
                 e[i] = radix_pair_entry<SG>(x[i], row[i], (uint32_t)(wb + i * 32), J, log2J);
+            }
         } else {
 #pragma unroll
             for (int i = 0; i < kRPer; ++i) {
+                if (i >= per) break;
                 const int64_t p = wb + i * 32;
                 e[i] = (p < n) ? __ldcs(in_e + p) : ~0ull;
             }
@@ -722,6 +735,7 @@ k_radix_down(const uint32_t* __restrict__ pair_x, const uint32_t* __restrict__ q
         const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
         for (int i = 0; i < kRPer; ++i) {
+            if (i >= per) break;
             const bool valid = e[i] != ~0ull;
             const uint32_t dg = valid ? ((uint32_t)(e[i] >> (32 + shift)) & dmask) : 0xffffffffu;
             const uint32_t peers = __match_any_sync(0xffffffffu, dg);
@@ -1625,36 +1639,57 @@ RadixPlan radix_plan(uint64_t R, int digit_bits) {
     return pl;
 }
 
-int64_t radix_tiles(int64_t npairs) {
-    const int64_t t = (npairs + kRTile - 1) / kRTile;
-    return t < 1 ? 1 : t;
+// Entries per thread of a tile: kRPer, or, for batches that leave tiles of half
+// that size within one wave of two CTAs per SM, as many as fill the wave (a
+// tile is one chain of loads, ranks and stores, so small tiles end sooner).
+// Measured on GB300, us of a deterministic training step of the Criteo-TB
+// shape, tiles of 8192 entries against these: batch 1600 85 / 73, 2500 95 / 83,
+// 4000 105 / 100, 8000 133 / 133; with the wave filled for larger batches too
+// 20011 208 / 211, 65536 515 / 536.
+static int radix_per(int64_t npairs, int sm_count) {
+    const int64_t wave = (int64_t)2 * sm_count * kRThreads;   // entries per unit of `per`
+    const int64_t per = (npairs + wave - 1) / wave;
+    if (per > kRPer / 2) return kRPer;
+    return (int)(per < kRMinPer ? kRMinPer : per);
+}
+
+// At least the tiles of any batch of up to npairs pairs (tiles of kRMinPer
+// entries per thread never exceed one wave).
+int64_t radix_tiles(int64_t npairs, int sm_count) {
+    const int64_t wave = (int64_t)2 * sm_count;
+    const int64_t waves = (npairs + wave * kRTile - 1) / (wave * kRTile);
+    return wave * (waves < 1 ? 1 : waves);
 }
 
 template <bool FIRST, bool SG>
 cudaError_t radix_pass(const SortedBuffers& sb, const unsigned long long* in,
                        unsigned long long* out, int64_t npairs, int J, int log2J,
-                       const RadixPlan& plan, int k, cudaStream_t st) {
-    const int ntiles = (int)radix_tiles(npairs);
+                       const RadixPlan& plan, int k, int sm_count, cudaStream_t st) {
+    const int per = radix_per(npairs, sm_count);
+    int ntiles = (int)((npairs + kRThreads * per - 1) / (kRThreads * per));
+    if (ntiles < 1) ntiles = 1;
     const int bits = plan.bits[k], shift = plan.shift[k];
     const int nd = 1 << bits;
-    cudaError_t e = launch_k(k_radix_up<FIRST, SG>, dim3(ntiles), dim3(kRThreads), 0, st,
-                             sb.pair_x, in, npairs, sb.stats, shift, bits, ntiles, sb.cnt);
+    const auto up = per == kRPer ? k_radix_up<FIRST, SG, true> : k_radix_up<FIRST, SG, false>;
+    const auto down = per == kRPer ? k_radix_down<FIRST, SG, true> : k_radix_down<FIRST, SG, false>;
+    cudaError_t e = launch_k(up, dim3(ntiles), dim3(kRThreads), 0, st,
+                             sb.pair_x, in, npairs, sb.stats, shift, bits, ntiles, per, sb.cnt);
     if (e != cudaSuccess) return e;
     e = launch_k(k_radix_colscan<FIRST>, dim3((nd + kRWarps - 1) / kRWarps), dim3(kRThreads), 0,
                  st, sb.cnt, ntiles, bits, sb.tot, sb.dstart, sb.done, sb.stats);
     if (e != cudaSuccess) return e;
     const size_t smem = radix_down_smem(nd);
     int per_sm = 1;   // (allows the shared memory)
-    e = resident_ctas(reinterpret_cast<const void*>(k_radix_down<FIRST, SG>), kRThreads, smem,
+    e = resident_ctas(reinterpret_cast<const void*>(down), kRThreads, smem,
                       &per_sm);
     if (e != cudaSuccess) return e;
-    return launch_k(k_radix_down<FIRST, SG>, dim3(ntiles), dim3(kRThreads), smem, st, sb.pair_x,
-                    sb.q_row, in, out, npairs, sb.stats, J, log2J, shift, bits, ntiles, sb.cnt,
+    return launch_k(down, dim3(ntiles), dim3(kRThreads), smem, st, sb.pair_x,
+                    sb.q_row, in, out, npairs, sb.stats, J, log2J, shift, bits, ntiles, per, sb.cnt,
                     sb.dstart);
 }
 
 cudaError_t launch_radix_sort(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
-                              const RadixPlan& plan, cudaStream_t st) {
+                              const RadixPlan& plan, int sm_count, cudaStream_t st) {
     const int log2J = (J & (J - 1)) == 0 ? ceil_log2(J) : -1;
     const unsigned long long* in = nullptr;
     for (int k = 0; k < plan.passes; ++k) {
@@ -1662,10 +1697,10 @@ cudaError_t launch_radix_sort(const SortedBuffers& sb, int64_t npairs, int J, ui
         unsigned long long* out = ((plan.passes - 1 - k) % 2 == 0) ? sb.sorted_e : sb.tmp_e;
         cudaError_t e;
         if (k == 0)
-            e = smask ? radix_pass<true, true>(sb, in, out, npairs, J, log2J, plan, k, st)
-                      : radix_pass<true, false>(sb, in, out, npairs, J, log2J, plan, k, st);
+            e = smask ? radix_pass<true, true>(sb, in, out, npairs, J, log2J, plan, k, sm_count, st)
+                      : radix_pass<true, false>(sb, in, out, npairs, J, log2J, plan, k, sm_count, st);
         else
-            e = radix_pass<false, false>(sb, in, out, npairs, J, log2J, plan, k, st);
+            e = radix_pass<false, false>(sb, in, out, npairs, J, log2J, plan, k, sm_count, st);
         if (e != cudaSuccess) return e;
         in = out;
     }
