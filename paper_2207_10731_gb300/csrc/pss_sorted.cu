@@ -6,21 +6,24 @@
 //              for an id outside its table;
 //   q_row[q]   output row b*T + t of the bag that holds id q;
 // Steps (all on the caller's stream):
-//   1. sort     a stable radix sort of the entries e = x << 32 | r by x, where
-//               r = row*J + j names the upstream-gradient chunk to add (with
-//               signed hashing, bit 31 of pair_x and of r carries the pair's
-//               sign, see pss_device.cuh); bad ids are dropped.  Entries of one
-//               bucket come out in pair order, so every later step sees the
-//               same sequence on every run;
-//   2. reduce   the sorted entries are cut into tasks of consecutive entries;
-//               the lanes of a task own columns of the block, add the chunks of
-//               each run of equal x with compensated (Kahan) fp32 sums, and add
-//               every run's sum once into the fp64 gradient accumulator
-//               g[G*x + z] -- one reduction per run and element instead of one
-//               per contribution, and no queue of reductions on a hot address.
-//               The distinct buckets (stats[1]) come from the counting sort's
-//               scan, or, after a radix sort, from the reduce.
-// With the touched update, k_mark_pairs lists the touched blocks from pair_x.
+//   1. sort     the entries e = x << 32 | r are grouped by x, where r = row*J + j
+//               names the upstream-gradient chunk to add (with signed hashing,
+//               bit 31 of pair_x and of r carries the pair's sign, see
+//               pss_device.cuh); bad ids are dropped.  Three ways: within
+//               segments of 8192 pairs (k_sort_local, most batches), all pairs
+//               by a counting sort, or by a stable radix sort (R > 2^22, and
+//               run-to-run identical bits: entries of one bucket come out in
+//               pair order);
+//   2. reduce   every warp or lane group takes consecutive entries, adds the
+//               chunks of each run of equal x with compensated (Kahan) fp32
+//               sums, and adds every run's sum once into the fp64 gradient
+//               accumulator g[G*x + z] -- one reduction per run and element
+//               instead of one per contribution, and no queue of reductions on
+//               a hot address.  The distinct buckets (stats[1]) come from the
+//               counting sort's scan, from the reduce after a radix sort, or
+//               from the reduce's marks after a counted local sort.
+// With the touched update, the local sort or k_mark_pairs lists the touched
+// blocks.
 // The optimizer pass over g follows (pss_kernels.cu).
 #include <climits>
 
