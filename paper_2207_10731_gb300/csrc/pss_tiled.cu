@@ -255,6 +255,7 @@ struct Sum<1> {
 // or id (1), mod P.
 struct FwdGeom {
     int wb, log2pw, log2pi, tiles_per_table;
+    bool by_table;        // tiles in the order of the tables, else of the bags
     uint64_t stepA[2], stepA2[2];
     uint64_t TJ;          // T * J: keys of consecutive ids
     uint64_t Gb;          // bytes between block starts
@@ -504,7 +505,8 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
 // own, and in tiles whose bags all hold one valid id a row costs one
 // shared-memory load, one multiply-add, one load and one store.  Tiles run
 // over the tables of a range of bags first, so that the rows that the GPU
-// writes at a time are one contiguous piece of the output.
+// writes at a time are one contiguous piece of the output (arrays beyond the
+// L2: over the bags of a table first, see kByTableMinM).
 template <int VW, int KC, typename XT, bool SG, int MODE>
 __global__ void __launch_bounds__(kThreads, fwd_min_ctas(VW, KC, MODE))
 k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ idx, int64_t nnz,
@@ -535,32 +537,41 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
     const int j0 = lane >> fg.log2pw;                // its first chunk
     const int lpb = 32 >> fg.log2pw;                 // lanes per bag
 
-    // tiles of this warp: tile number = r * T + t (below 2^30, checked by the
-    // launcher), advanced without divisions, and with it the place of the
-    // lane's bag in the offsets
+    // tiles of this warp: tile number = r * T + t, or t * tpt + r (below 2^30,
+    // checked by the launcher), advanced without divisions, and with it the
+    // place of the lane's bag in the offsets
+    const bool by_table = fg.by_table;
     const int nwarps = (int)gridDim.x * kWarps;
-    const int step_r = nwarps / p.T, step_t = nwarps - step_r * p.T;
+    const int inner = by_table ? tpt : p.T;
+    const int step_out = nwarps / inner, step_in = nwarps - step_out * inner;
+    const int step_t = by_table ? step_out : step_in, step_r = by_table ? step_in : step_out;
     const int64_t step_o = (int64_t)step_t * B + (int64_t)step_r * wb;
-    const int64_t wrap_o = wb - (int64_t)p.T * B;
-    int r = ((int)blockIdx.x * kWarps + warp) / p.T;
-    int t = ((int)blockIdx.x * kWarps + warp) - r * p.T;
-    if (r >= tpt) return;
+    const int64_t wrap_o = by_table ? B - (int64_t)tpt * wb : wb - (int64_t)p.T * B;
+    const int tile0 = (int)blockIdx.x * kWarps + warp, out0 = tile0 / inner;
+    int t = by_table ? out0 : tile0 - out0 * inner;
+    int r = by_table ? tile0 - out0 * inner : out0;
+    if (t >= p.T || r >= tpt) return;
     const int64_t* po = off + (int64_t)t * B + b_lo + (int64_t)r * wb + bag;
     const int64_t nbags = b_hi - b_lo;
     auto advance = [&](int& tt, int& rr) {
         tt += step_t;
         rr += step_r;
         po += step_o;
-        if (tt >= p.T) {
-            tt -= p.T;
-            ++rr;
+        if (by_table ? rr >= tpt : tt >= p.T) {
+            if (by_table) {
+                rr -= tpt;
+                ++tt;
+            } else {
+                tt -= p.T;
+                ++rr;
+            }
             po += wrap_o;
         }
     };
-    // offsets of this lane's bag of tile row rr at po: a zero-length bag past the end
-    auto load_offsets = [&](int rr, int64_t& q0, int64_t& q1) {
+    // offsets of this lane's bag of tile (tt, rr) at po: a zero-length bag past the end
+    auto load_offsets = [&](int tt, int rr, int64_t& q0, int64_t& q1) {
         q0 = q1 = 0;
-        if (bag < wb && (int64_t)rr * wb + bag < nbags) {
+        if (bag < wb && tt < p.T && (int64_t)rr * wb + bag < nbags) {
             q0 = __ldg(po);
             q1 = __ldg(po + 1);
         }
@@ -571,17 +582,17 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
     };
 
     int64_t q0, q1, q0n, q1n;
-    load_offsets(r, q0, q1);
+    load_offsets(t, r, q0, q1);
     int t1 = t, r1 = r;
     advance(t1, r1);
-    load_offsets(r1, q0n, q1n);
+    load_offsets(t1, r1, q0n, q1n);
     int64_t id = load_id(q0, q1);
-    while (r < tpt) {
+    while (t < p.T && r < tpt) {
         int t2 = t1, r2 = r1;
         advance(t2, r2);
         const int64_t idn = load_id(q0n, q1n);
         int64_t q0m, q1m;
-        load_offsets(r2, q0m, q1m);
+        load_offsets(t2, r2, q0m, q1m);
 
         const int64_t b0 = b_lo + (int64_t)r * wb;
         const int nb = (int)((b_hi - b0) < wb ? (b_hi - b0) : wb);
@@ -817,6 +828,14 @@ size_t tile_smem(const TileGeom& g, const DevParams& p, size_t xbytes) {
     return sizeof(int64_t) * (size_t)(g.tb + 1) + xbytes * (size_t)g.qc * (size_t)p.J;
 }
 
+// Arrays from this many elements on take their tiles table by table: beyond the
+// L2 the blocks of one table's hot ids stay in it better than those of all
+// tables at once; smaller arrays take them bag by bag, whose rows HBM writes
+// better.  Measured on GB300, us per serving forward of 65536 rows, bag by bag
+// against table by table: M = 2^20 144 / 157 (an earlier kernel), 2^24 182 /
+// 178, 2^25 195 / 191, 2^26 211 / 199, 2^28 220 / 204.
+constexpr int64_t kByTableMinM = int64_t(1) << 24;
+
 // Bags per tile of the forward: a multiple of the lane groups (and of 4), at
 // most kWarpPairs staged pairs and 16 bags or 4 per lane group, chosen so that
 // the warps' rounds of tiles waste least: rounds * (wb + 8) is smallest, a
@@ -861,6 +880,7 @@ cudaError_t fwd_mode(const DevParams& p, const RowLayout& lay, const int64_t* id
     // (room for the stride past the last tile)
     if (ntiles >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;
     fg.tiles_per_table = (int)tpt;
+    fg.by_table = p.M >= kByTableMinM;
     fg.TJ = (uint64_t)p.T * (uint64_t)p.J;
     fg.Gb = (uint64_t)p.G * sizeof(float);
     for (int k = 0; k < 2; ++k) {
