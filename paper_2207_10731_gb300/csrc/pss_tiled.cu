@@ -21,6 +21,7 @@
 
 #include "pss_device.cuh"
 #include "pss_internal.h"
+#include "pss_tiles.h"
 
 namespace pss {
 namespace {
@@ -122,8 +123,6 @@ __device__ __forceinline__ typename V::T gather(const float* __restrict__ wz, ui
 // stages it in its own slice of shared memory, so warps never wait for each
 // other (no CTA-wide barrier): the lanes hash the tile's (id, chunk) pairs
 // 32 at a time, then the lane groups gather and sum-pool their bags.
-constexpr int kWarpPairs = 512;   // staged pairs per warp and round
-constexpr int kMaxTileBags = 32;  // bags per tile at most: one lane each
 constexpr int kIdU = 4;           // ids in flight per lane while a window is hashed
 
 
@@ -836,31 +835,6 @@ size_t tile_smem(const TileGeom& g, const DevParams& p, size_t xbytes) {
 // 178, 2^25 195 / 191, 2^26 211 / 199, 2^28 220 / 204.
 constexpr int64_t kByTableMinM = int64_t(1) << 24;
 
-// Bags per tile of the forward: a multiple of the lane groups (and of 4), at
-// most kWarpPairs staged pairs and 16 bags or 4 per lane group, chosen so that
-// the warps' rounds of tiles waste least: rounds * (wb + 8) is smallest, a
-// tile's fixed work being about that of 8 bags.  Measured on GB300, us per
-// forward at 4, 8, 12, 16, 24 and 32 bags: Criteo-TB shape 227, 158, 150, 153,
-// 156, 156; multi-hot 326, 310, 303, 294, 298, 314; 16-float rows (batch 16384,
-// 8 lane groups) 36, 25, 18, 14, 11, 9.6.
-int tile_bags(const DevParams& p, const RowLayout& lay, int64_t rows, int64_t warps) {
-    const int ng = 32 >> lay.log2gs;
-    const int step = ng > 4 ? ng : 4;
-    int best = step;
-    int64_t best_cost = INT64_MAX;
-    const int most = 4 * ng > 16 ? 4 * ng : 16;
-    for (int wb = step; wb <= most; wb += step) {
-        if (wb > step && wb * p.J > kWarpPairs) break;
-        const int64_t tiles = (int64_t)p.T * ((rows + wb - 1) / wb);
-        const int64_t cost = ((tiles + warps - 1) / warps) * (wb + 8);
-        if (cost <= best_cost) {
-            best_cost = cost;
-            best = wb;
-        }
-    }
-    return best;
-}
-
 template <int VW, int KC, typename XT, bool SG, int MODE>
 cudaError_t fwd_mode(const DevParams& p, const RowLayout& lay, const int64_t* idx, int64_t nnz,
                      const int64_t* off, int64_t B, const float* w, float* out, DevError* err,
@@ -871,7 +845,8 @@ cudaError_t fwd_mode(const DevParams& p, const RowLayout& lay, const int64_t* id
     const int64_t rows = b_hi - b_lo;
     const int max_grid = grid_for(kern, sm_count, INT32_MAX, smem);
     FwdGeom fg;
-    fg.wb = tile_bags(p, lay, rows, (int64_t)max_grid * kWarps);
+    fg.wb = tile_bags(p.T, p.J, lay.log2gs, rows, (int64_t)max_grid * kWarps);
+    if (fg.wb > kMaxTileBags) return cudaErrorInvalidValue;   // a bag without a lane
     fg.log2pw = ceil_log2(fg.wb);
     fg.log2pi = 0;
     while (fg.log2pi < 5 && (2 << fg.log2pi) * p.J <= kWarpPairs) ++fg.log2pi;
