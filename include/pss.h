@@ -29,7 +29,8 @@
  * Batch layout (all int64, CSR, TABLE-MAJOR bags):
  *   bag (t, b) is slot s = t*B + b and owns indices[offsets[s] .. offsets[s+1]);
  *   offsets has T*B + 1 entries, non-decreasing, offsets[0] >= 0,
- *   offsets[T*B] <= nnz.  Pooled outputs and upstream gradients are fp32,
+ *   offsets[T*B] <= nnz; ids before the first bag and after the last are in no
+ *   bag and add nothing.  Pooled outputs and upstream gradients are fp32,
  *   row-major [B][T][d] (the DLRM concatenation order).
  *
  * Memory and streams:
@@ -51,7 +52,9 @@
  * arguments are rejected on the host before any work is queued.  An id outside
  * [0, n_t) cannot be seen on the host; the device skips that id (it contributes
  * nothing) and records the smallest such position in a device error word,
- * which pss_get_error() reads and clears.
+ * which pss_get_error() reads and clears.  Malformed offsets are recorded there
+ * too; the rows and gradients of such a batch are unspecified near them, but
+ * nothing is read or written outside the batch's buffers.
  */
 #ifndef PSS_H_
 #define PSS_H_

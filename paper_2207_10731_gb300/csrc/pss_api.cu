@@ -922,6 +922,8 @@ static pss_status ensure_seen(pss_handle* h, cudaStream_t st) {
 // radix sort); with `touch`, also list the touched blocks.
 static pss_status sort_pairs(pss_handle* h, bool touch, LocalSort local, cudaStream_t st) {
     const int64_t npairs = h->last_nnz * (int64_t)h->dp.J;
+    h->sb.R = (uint32_t)h->dp.R;   // (below 2^32, and so are the rows: sorted_supported)
+    h->sb.rows = (uint32_t)(h->dp.T * h->last_B);
     poll_stats(h);
     if (local != kLocalNo) {
         // grouped within segments only: the distinct buckets are marked and

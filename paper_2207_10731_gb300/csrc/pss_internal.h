@@ -82,6 +82,7 @@ int64_t radix_tiles(int64_t npairs, int sm_count);   // tiles of a pass of up to
 struct SortedBuffers {
     uint32_t* pair_x;             // nnz*J buckets written by the forward (0xffffffff: bad id)
     uint32_t* q_row;              // nnz output rows b*T + t written by the forward
+    uint32_t R, rows;             // block starts, and output rows of the batch
     unsigned long long* sorted_e; // nnz*J entries (x << 32 | row*J + j), grouped by x
     unsigned long long* stats;    // [0] valid pairs, [1] distinct buckets
     float* bnd;                   // window reduce: boundary records, 64 floats per range
@@ -168,7 +169,7 @@ cudaError_t launch_locations(const DevParams& p, const int64_t* idx, int64_t nnz
 // Forward of the bags of batch rows [b_lo, b_hi) of every table (0 <= b_lo <
 // b_hi <= B; out, idx and off are the whole batch's); when pair_x / q_row are
 // given it also writes those bags' pairs' buckets and ids' output rows for the
-// sorted backward path.
+// sorted backward path (0xffffffff for the ids that lie in no bag).
 cudaError_t launch_forward(const DevParams& p, const RowLayout& lay, const int64_t* idx,
                            int64_t nnz, const int64_t* off, int64_t B, const float* w, float* out,
                            DevError* err, uint32_t* pair_x, uint32_t* q_row, int64_t b_lo,

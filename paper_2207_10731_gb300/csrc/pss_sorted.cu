@@ -41,6 +41,30 @@ constexpr int kRU = 4;            // entries in flight per group (summed as a tr
                                   // all continue the current run)
 static_assert(kRU == 4, "the reduce sums kRU = 4 entries as a tree");
 
+// What the forward left for the sorts.  Every pair is written by a batch whose
+// offsets are in order; where malformed ones leave values of another batch (or
+// none), the bounds here keep buckets and rows inside the buffers.
+struct Pairs {
+    const uint32_t* x;        // pair_x and q_row of SortedBuffers
+    const uint32_t* row;
+    uint32_t R, rows;
+    explicit Pairs(const SortedBuffers& sb)
+        : x(sb.pair_x), row(sb.q_row), R(sb.R), rows(sb.rows) {}
+    // Bucket, with its sign, of pair p; kBad past the end.
+    __device__ __forceinline__ uint32_t at(int64_t p, int64_t npairs) const {
+        return p < npairs ? __ldg(x + p) : kBad;
+    }
+    // Not a bad id's (kBad is above every bucket, also without its sign).
+    __device__ __forceinline__ bool valid(uint32_t v, uint32_t smask) const {
+        return (v & ~smask) < R;
+    }
+    // Output row of id q when `valid`, else 0; clamp it when every load is under way.
+    __device__ __forceinline__ uint32_t row_of(uint32_t q, bool valid) const {
+        return valid ? __ldg(row + q) : 0u;
+    }
+    __device__ __forceinline__ uint32_t clamp(uint32_t r) const { return min(r, rows - 1u); }
+};
+
 // Block-wide exclusive scan of one value per thread (kScanThreads threads).
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s_warp,
                                                          uint32_t* total) {
@@ -196,8 +220,7 @@ __device__ __forceinline__ void seg_table_init(uint32_t* s_key, uint32_t* s_val)
 
 // cnt[x] += number of valid pairs with bucket x (without its sign).
 __global__ void __launch_bounds__(kSegThreads)
-k_sort_count(const uint32_t* __restrict__ pair_x, int64_t npairs, uint32_t smask,
-             uint32_t* __restrict__ cnt) {
+k_sort_count(const Pairs pairs, int64_t npairs, uint32_t smask, uint32_t* __restrict__ cnt) {
     pdl_prologue();
     __shared__ uint32_t s_key[kSegSlots];
     __shared__ uint32_t s_val[kSegSlots];
@@ -209,12 +232,12 @@ k_sort_count(const uint32_t* __restrict__ pair_x, int64_t npairs, uint32_t smask
 #pragma unroll
         for (int i = 0; i < kSegPer; ++i) {
             const int64_t p = p0 + i * kSegThreads + threadIdx.x;
-            x[i] = (p < npairs) ? __ldg(pair_x + p) : kBad;
+            x[i] = pairs.at(p, npairs);
         }
         __syncthreads();   // the previous segment's table is clear
 #pragma unroll
         for (int i = 0; i < kSegPer; ++i)
-            hr[i] = (x[i] != kBad) ? seg_insert(s_key, s_val, x[i] & ~smask) : 0u;
+            hr[i] = pairs.valid(x[i], smask) ? seg_insert(s_key, s_val, x[i] & ~smask) : 0u;
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < kSegSlots / kSegThreads; ++k) {
@@ -226,7 +249,7 @@ k_sort_count(const uint32_t* __restrict__ pair_x, int64_t npairs, uint32_t smask
         // each thread clears the slots of its own pairs
 #pragma unroll
         for (int i = 0; i < kSegPer; ++i)
-            if (x[i] != kBad) {
+            if (pairs.valid(x[i], smask)) {
                 s_key[hr[i] & 0xffffu] = kEmpty;
                 s_val[hr[i] & 0xffffu] = 0u;
             }
@@ -242,8 +265,7 @@ k_sort_count(const uint32_t* __restrict__ pair_x, int64_t npairs, uint32_t smask
 // sorted_e[slot] = x << 32 | row*J + j.
 template <bool SG>
 __global__ void __launch_bounds__(kSegThreads)
-k_sort_scatter(const uint32_t* __restrict__ pair_x, int64_t npairs, const uint32_t* __restrict__ q_row,
-               int J, int log2J, uint32_t* __restrict__ start,
+k_sort_scatter(const Pairs pairs, int64_t npairs, int J, int log2J, uint32_t* __restrict__ start,
                unsigned long long* __restrict__ sorted_e) {
     pdl_prologue();
     __shared__ uint32_t s_key[kSegSlots];
@@ -256,7 +278,7 @@ k_sort_scatter(const uint32_t* __restrict__ pair_x, int64_t npairs, const uint32
 #pragma unroll
         for (int i = 0; i < kSegPer; ++i) {
             const int64_t p = p0 + i * kSegThreads + threadIdx.x;
-            x[i] = (p < npairs) ? __ldg(pair_x + p) : kBad;
+            x[i] = pairs.at(p, npairs);
         }
         // loads that do not depend on the table go first, so they overlap it
 #pragma unroll
@@ -264,8 +286,10 @@ k_sort_scatter(const uint32_t* __restrict__ pair_x, int64_t npairs, const uint32
             const uint32_t pp = (uint32_t)(p0 + i * kSegThreads + threadIdx.x);  // npairs < 2^32 here
             const uint32_t q = (log2J >= 0) ? (pp >> log2J) : pp / (uint32_t)J;
             e[i] = pp - q * (uint32_t)J;
-            if (x[i] != kBad) {
-                e[i] += __ldg(q_row + q) * (uint32_t)J;
+            if (!pairs.valid(x[i], SG ? 0x80000000u : 0u)) {
+                x[i] = kBad;
+            } else {
+                e[i] += pairs.clamp(pairs.row_of(q, true)) * (uint32_t)J;
                 if (SG) {
                     // signed hashing: the sign moves to bit 31 of the entry's low word
                     e[i] |= x[i] & 0x80000000u;
@@ -358,11 +382,11 @@ __host__ __device__ constexpr size_t local_smem(bool touch) {
 // (k_count_seen adds to them).
 template <bool SG, bool TOUCH>
 __global__ void __launch_bounds__(kLSThreads, 2)
-k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
-             const uint32_t* __restrict__ q_row, int J, int log2J,
+k_sort_local(const Pairs pairs, int64_t npairs, int J, int log2J,
              unsigned long long* __restrict__ sorted_e, uint32_t* __restrict__ segn,
              Touched tc, unsigned long long* __restrict__ stats) {
     pdl_prologue();
+    constexpr uint32_t kSign = SG ? 0x80000000u : 0u;
     extern __shared__ __align__(16) unsigned char ls_smem[];
     uint32_t* s_w = reinterpret_cast<uint32_t*>(ls_smem);                               // [kLSWords]
     unsigned long long* s_e = reinterpret_cast<unsigned long long*>(ls_smem);           // [kLS]
@@ -379,7 +403,7 @@ k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
 #pragma unroll
         for (int i = 0; i < kLSPer; ++i) {
             const int64_t p = p0 + i * kLSThreads + tid;
-            x[i] = (p < npairs) ? __ldg(pair_x + p) : kBad;
+            x[i] = pairs.at(p, npairs);
         }
 #pragma unroll
         for (int k = 0; k < kLSWords / 4 / kLSThreads; ++k)
@@ -393,7 +417,9 @@ k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
 #pragma unroll
         for (int i = 0; i < kLSPer; ++i) {
             const uint32_t sl = slot_of(x[i]), sh = (sl & 1u) * 16u;
-            pos[i] = (x[i] != kBad) ? (atomicAdd(s_w + (sl >> 1), 1u << sh) >> sh) & 0xffffu : 0u;
+            pos[i] = pairs.valid(x[i], kSign)
+                         ? (atomicAdd(s_w + (sl >> 1), 1u << sh) >> sh) & 0xffffu
+                         : 0u;
         }
         __syncthreads();
         // slot starts: exclusive prefix of the counts in the order (thread, k)
@@ -420,7 +446,7 @@ k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
             const uint32_t pp = (uint32_t)(p0 + i * kLSThreads + tid);   // npairs < 2^32 here
             const uint32_t q = (log2J >= 0) ? (pp >> log2J) : pp / (uint32_t)J;
             e[i] = pp - q * (uint32_t)J;
-            if (x[i] != kBad) e[i] += __ldg(q_row + q) * (uint32_t)J;
+            e[i] += pairs.clamp(pairs.row_of(q, pairs.valid(x[i], kSign))) * (uint32_t)J;
         }
         __syncthreads();
 #pragma unroll
@@ -431,7 +457,7 @@ k_sort_local(const uint32_t* __restrict__ pair_x, int64_t npairs,
         __syncthreads();   // every place is known: the entries take the counters' place
 #pragma unroll
         for (int i = 0; i < kLSPer; ++i) {
-            if (x[i] == kBad) continue;
+            if (!pairs.valid(x[i], kSign)) continue;
             // signed hashing: the sign moves to bit 31 of the entry's low word
             const uint32_t xi = SG ? x[i] & 0x7fffffffu : x[i];
             const uint32_t ei = SG ? e[i] | (x[i] & 0x80000000u) : e[i];
@@ -521,13 +547,13 @@ __device__ __forceinline__ uint32_t rblock_exclusive_scan(uint32_t v, uint32_t* 
     return pre + x - v;
 }
 
-// Entry of pair p from its bucket x (kBad for a bad id) and its id's output
-// row: x << 32 | row*J + j, or ~0 when invalid.  Buckets are below 2^32 - 1,
+// Entry of pair p from its bucket x (and whether it is a valid one) and its id's
+// output row: x << 32 | row*J + j, or ~0 when invalid.  Buckets are below 2^32 - 1,
 // so an all-ones entry is never valid.
 template <bool SG>
-__device__ __forceinline__ unsigned long long radix_pair_entry(uint32_t x, uint32_t row,
+__device__ __forceinline__ unsigned long long radix_pair_entry(bool valid, uint32_t x, uint32_t row,
                                                                uint32_t p, int J, int log2J) {
-    if (x == kBad) return ~0ull;
+    if (!valid) return ~0ull;
     const uint32_t q = (log2J >= 0) ? (p >> log2J) : p / (uint32_t)J;
     uint32_t r = row * (uint32_t)J + (p - q * (uint32_t)J);
     if (SG) {
@@ -550,7 +576,7 @@ __device__ __forceinline__ int64_t radix_count(int64_t npairs,
 // of its nd counts, zeros included).
 template <bool FIRST, bool SG, bool FULL>
 __global__ void __launch_bounds__(kRThreads)
-k_radix_up(const uint32_t* __restrict__ pair_x, const unsigned long long* __restrict__ in_e,
+k_radix_up(const Pairs pairs, const unsigned long long* __restrict__ in_e,
            int64_t npairs, const unsigned long long* __restrict__ stats, int shift, int bits,
            int ntiles, int per_arg, uint32_t* __restrict__ cnt) {
     pdl_prologue();
@@ -570,8 +596,9 @@ k_radix_up(const uint32_t* __restrict__ pair_x, const unsigned long long* __rest
         if (i >= per) break;
         const int64_t p = t0 + (int64_t)i * kRThreads + threadIdx.x;
         if (FIRST) {
-            hi[i] = (p < n) ? __ldg(pair_x + p) : kBad;
-            if (SG && hi[i] != kBad) hi[i] &= 0x7fffffffu;
+            hi[i] = pairs.at(p, n);
+            if (!pairs.valid(hi[i], SG ? 0x80000000u : 0u)) hi[i] = kBad;
+            else if (SG) hi[i] &= 0x7fffffffu;
         } else {
             hi[i] = (p < n) ? reinterpret_cast<const uint32_t*>(in_e)[2 * p + 1] : kBad;
         }
@@ -670,8 +697,8 @@ __host__ __device__ constexpr size_t radix_down_smem(int nd) {
 // down: one tile per CTA (see the section comment).
 template <bool FIRST, bool SG, bool FULL>
 __global__ void __launch_bounds__(kRThreads, 2)
-k_radix_down(const uint32_t* __restrict__ pair_x, const uint32_t* __restrict__ q_row,
-             const unsigned long long* __restrict__ in_e, unsigned long long* __restrict__ out_e,
+k_radix_down(const Pairs pairs, const unsigned long long* __restrict__ in_e,
+             unsigned long long* __restrict__ out_e,
              int64_t npairs, const unsigned long long* __restrict__ stats, int J, int log2J,
              int shift, int bits, int ntiles, int per_arg, const uint32_t* __restrict__ cnt,
              const uint32_t* __restrict__ dstart) {
@@ -707,19 +734,21 @@ k_radix_down(const uint32_t* __restrict__ pair_x, const uint32_t* __restrict__ q
             for (int i = 0; i < kRPer; ++i) {
                 if (i >= per) break;
                 const int64_t p = wb + i * 32;
-                x[i] = (p < n) ? __ldg(pair_x + p) : kBad;
+                x[i] = pairs.at(p, n);
             }
 #pragma unroll
             for (int i = 0; i < kRPer; ++i) {
                 if (i >= per) break;
                 const uint32_t pp = (uint32_t)(wb + i * 32);   // npairs < 2^32 here
                 const uint32_t q = (log2J >= 0) ? (pp >> log2J) : pp / (uint32_t)J;
-                row[i] = (wb + i * 32 < n) ? __ldg(q_row + q) : 0u;
+                row[i] = pairs.row_of(q, wb + i * 32 < n);
             }
 #pragma unroll
             for (int i = 0; i < kRPer; ++i) {
                 if (i >= per) break;
-                e[i] = radix_pair_entry<SG>(x[i], row[i], (uint32_t)(wb + i * 32), J, log2J);
+                e[i] = radix_pair_entry<SG>(pairs.valid(x[i], SG ? 0x80000000u : 0u), x[i],
+                                            pairs.clamp(row[i]),
+                                            (uint32_t)(wb + i * 32), J, log2J);
             }
         } else {
 #pragma unroll
@@ -813,7 +842,7 @@ constexpr int kMarkPer = 16;                          // pairs per thread and ch
 constexpr int kMarkChunk = kThreads * kMarkPer;
 
 __global__ void __launch_bounds__(kThreads)
-k_mark_pairs(const uint32_t* __restrict__ pair_x, int64_t npairs, uint32_t smask, Touched tc) {
+k_mark_pairs(const Pairs pairs, int64_t npairs, uint32_t smask, Touched tc) {
     pdl_prologue();
     __shared__ uint32_t s_new[kMarkChunk];
     __shared__ uint32_t s_n;
@@ -826,12 +855,13 @@ k_mark_pairs(const uint32_t* __restrict__ pair_x, int64_t npairs, uint32_t smask
 #pragma unroll
         for (int i = 0; i < kMarkPer; ++i) {
             const int64_t p = c * kMarkChunk + i * kThreads + threadIdx.x;
-            x[i] = (p < npairs) ? __ldg(pair_x + p) : kBad;
+            x[i] = pairs.at(p, npairs);
         }
 #pragma unroll
         for (int i = 0; i < kMarkPer; ++i) {
-            if (x[i] != kBad) x[i] &= ~smask;
-            word[i] = (x[i] != kBad) ? __ldcg(tc.bitmap + (x[i] >> 5)) : ~0u;
+            const bool valid = pairs.valid(x[i], smask);
+            x[i] &= ~smask;
+            word[i] = valid ? __ldcg(tc.bitmap + (x[i] >> 5)) : ~0u;
         }
 #pragma unroll
         for (int i = 0; i < kMarkPer; ++i) {
@@ -1676,7 +1706,7 @@ cudaError_t radix_pass(const SortedBuffers& sb, const unsigned long long* in,
     const auto up = per == kRPer ? k_radix_up<FIRST, SG, true> : k_radix_up<FIRST, SG, false>;
     const auto down = per == kRPer ? k_radix_down<FIRST, SG, true> : k_radix_down<FIRST, SG, false>;
     cudaError_t e = launch_k(up, dim3(ntiles), dim3(kRThreads), 0, st,
-                             sb.pair_x, in, npairs, sb.stats, shift, bits, ntiles, per, sb.cnt);
+                             Pairs(sb), in, npairs, sb.stats, shift, bits, ntiles, per, sb.cnt);
     if (e != cudaSuccess) return e;
     e = launch_k(k_radix_colscan<FIRST>, dim3((nd + kRWarps - 1) / kRWarps), dim3(kRThreads), 0,
                  st, sb.cnt, ntiles, bits, sb.tot, sb.dstart, sb.done, sb.stats);
@@ -1686,9 +1716,8 @@ cudaError_t radix_pass(const SortedBuffers& sb, const unsigned long long* in,
     e = resident_ctas(reinterpret_cast<const void*>(down), kRThreads, smem,
                       &per_sm);
     if (e != cudaSuccess) return e;
-    return launch_k(down, dim3(ntiles), dim3(kRThreads), smem, st, sb.pair_x,
-                    sb.q_row, in, out, npairs, sb.stats, J, log2J, shift, bits, ntiles, per, sb.cnt,
-                    sb.dstart);
+    return launch_k(down, dim3(ntiles), dim3(kRThreads), smem, st, Pairs(sb), in, out,
+                    npairs, sb.stats, J, log2J, shift, bits, ntiles, per, sb.cnt, sb.dstart);
 }
 
 cudaError_t launch_radix_sort(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
@@ -1729,19 +1758,19 @@ cudaError_t launch_sorted_scatter(const SortedBuffers& sb, int64_t npairs, int J
     const int64_t nseg = (npairs + kSeg - 1) / kSeg;
     if (smask) {
         const int grid = grid_for(k_sort_scatter<true>, sm_count, nseg);
-        return launch_k(k_sort_scatter<true>, dim3(grid), dim3(kSegThreads), 0, st, sb.pair_x,
-                        npairs, sb.q_row, J, log2J, sb.start, sb.sorted_e);
+        return launch_k(k_sort_scatter<true>, dim3(grid), dim3(kSegThreads), 0, st, Pairs(sb),
+                        npairs, J, log2J, sb.start, sb.sorted_e);
     }
     const int grid = grid_for(k_sort_scatter<false>, sm_count, nseg);
-    return launch_k(k_sort_scatter<false>, dim3(grid), dim3(kSegThreads), 0, st, sb.pair_x, npairs,
-                    sb.q_row, J, log2J, sb.start, sb.sorted_e);
+    return launch_k(k_sort_scatter<false>, dim3(grid), dim3(kSegThreads), 0, st, Pairs(sb), npairs,
+                    J, log2J, sb.start, sb.sorted_e);
 }
 
 cudaError_t launch_sorted_count(const SortedBuffers& sb, int64_t npairs, uint32_t smask,
                                 int sm_count, cudaStream_t st) {
     const int64_t nseg = (npairs + kSeg - 1) / kSeg;
     const int grid = grid_for(k_sort_count, sm_count, nseg);
-    return launch_k(k_sort_count, dim3(grid), dim3(kSegThreads), 0, st, sb.pair_x, npairs, smask,
+    return launch_k(k_sort_count, dim3(grid), dim3(kSegThreads), 0, st, Pairs(sb), npairs, smask,
                     sb.ccnt);
 }
 
@@ -1749,7 +1778,7 @@ cudaError_t launch_mark_pairs(const SortedBuffers& sb, int64_t npairs, uint32_t 
                               const Touched& touched, int sm_count, cudaStream_t st) {
     const int64_t chunks = (npairs + kMarkChunk - 1) / kMarkChunk;
     const int grid = grid_for(k_mark_pairs, sm_count, chunks);
-    return launch_k(k_mark_pairs, dim3(grid), dim3(kThreads), 0, st, sb.pair_x, npairs, smask,
+    return launch_k(k_mark_pairs, dim3(grid), dim3(kThreads), 0, st, Pairs(sb), npairs, smask,
                     touched);
 }
 
@@ -1841,7 +1870,7 @@ cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, ui
     if (e != cudaSuccess) return e;
     const int64_t nseg = local_segments(npairs), most = (int64_t)sm_count * per_sm;
     return launch_k(kern, dim3((unsigned)(nseg < most ? nseg : most)), dim3(kLSThreads), smem, st,
-                    sb.pair_x, npairs, sb.q_row, J, log2J, sb.sorted_e, sb.segn,
+                    Pairs(sb), npairs, J, log2J, sb.sorted_e, sb.segn,
                     touched ? *touched : Touched{}, sb.stats);
 }
 

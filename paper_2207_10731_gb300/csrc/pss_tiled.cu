@@ -497,6 +497,29 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
     }
 }
 
+// The two cases in which an id has no pair, whose buckets become Invalid.  Both
+// are rare and kept out of the forward's code: inlined, they cost the one-id
+// variant 3 us of 155 (Criteo-TB shape).
+// (1) Ids before the first bag and after the last: a and b are the batch's first
+// and last offset, and one warp of every CTA calls this.
+__device__ __noinline__ void drop_unused(int64_t a, int64_t b, int64_t nnz, int J,
+                                         uint32_t* __restrict__ pair_x, int lane) {
+    const int64_t head = (a < nnz ? a : nnz) * J;
+    const int64_t tail = (b < 0 ? 0 : b) * J;
+    const int64_t stride = (int64_t)gridDim.x * 32, k0 = (int64_t)blockIdx.x * 32 + lane;
+    for (int64_t k = k0; k < head; k += stride) pair_x[k] = Invalid<uint32_t>::v;
+    for (int64_t k = tail + k0; k < nnz * J; k += stride) pair_x[k] = Invalid<uint32_t>::v;
+}
+// (2) The ids [qa, qb) of a tile with malformed offsets, as far as those tell
+// them (the sorts check the bounds of what else malformed offsets leave; ranges
+// that may enclose the whole batch, for every such tile, are left).
+__device__ __noinline__ void drop_tile(int64_t qa, int64_t qb, int64_t nnz, int J,
+                                       uint32_t* __restrict__ pair_x, int lane) {
+    constexpr int64_t kMost = 1 << 16;   // pairs
+    if (qa < 0 || qb > nnz || (qb - qa) * J > kMost) return;
+    for (int64_t k = qa * J + lane; k < qb * J; k += 32) pair_x[k] = Invalid<uint32_t>::v;
+}
+
 // What bounds it with one-id bags: the pooled rows' stores to HBM at d = 128
 // (one 16-byte load and store per lane and row), and the latency of the chain
 // offsets -> ids -> hash -> blocks behind them.  So a warp loads the offsets
@@ -585,6 +608,10 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
     int t1 = t, r1 = r;
     advance(t1, r1);
     load_offsets(t1, r1, q0n, q1n);
+    if (pair_x && warp == 0 && b_lo == 0) {   // (these loads arrive with the tile's offsets)
+        const int64_t a = __ldg(off), b = __ldg(off + (int64_t)p.T * B);
+        if (a > 0 || b < nnz) drop_unused(a, b, nnz, J, pair_x, lane);
+    }
     int64_t id = load_id(q0, q1);
     while (t < p.T && r < tpt) {
         int t2 = t1, r2 = r1;
@@ -614,6 +641,9 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
                         for (int i = 0; i < VW; ++i) V::set(z, i, 0.f);
                         V::stcs(obase + bi * ostride + col.e[k], z);
                     }
+                if (pair_x)
+                    drop_tile(__shfl_sync(0xffffffffu, q0, 0), __shfl_sync(0xffffffffu, q1, nb - 1),
+                              nnz, J, pair_x, lane);
             } else {
                 forward_bags<VW, KC, XT, SG, MODE == kFwdLong>(
                     p, fg, idx, tJ, card, q0, q1, nb, s_x, wz, col, obase, ostride, row0, err,
