@@ -92,12 +92,16 @@ typedef enum {
      * scheduling, so low-order bits may differ between runs (within the
      * accumulation bound; dyadic inputs give identical bits).  The sorted path
      * groups the contributions by location and sums each location's run once
-     * (see PSS_OPT_DETERMINISTIC for its order).  PSS_PATH_AUTO takes the
-     * sorted path when the batch adds at least 3,500,000 elements (nnz * J *
-     * L) where the local sort serves it (PSS_OPT_SORT_SCOPE; blocks of L >= 8
-     * elements, fp64 accumulation); otherwise 5,000,000 with blocks of L >= 32
-     * elements and 10,000,000 with shorter ones; the atomic one below
-     * (crossovers measured on GB300; M does not move them). */
+     * (see PSS_OPT_DETERMINISTIC for its order), in fp32 with compensation,
+     * before the sums meet in fp64.  PSS_PATH_AUTO takes the
+     * sorted path when the batch adds at least 5,000,000 elements (nnz * J *
+     * L) with blocks of L >= 32 elements, 10,000,000 with shorter ones, the
+     * atomic path below (crossovers measured on GB300; M does not move them).
+     * From 3,500,000 elements on, AUTO already sorts the batches whose contributions it can all add in fp64,
+     * as the atomic path does: those that the local sort serves
+     * (PSS_OPT_SORT_SCOPE), with Z = 32 (d a multiple of 32, 16-byte aligned
+     * upstream gradient) or with L = 8 or 16 (chunks that tile the rows, dense
+     * update), and fp64 accumulation. */
     PSS_OPT_BACKWARD_PATH = 1,
     /* How the Adagrad step visits M: every element (PSS_UPDATE_DENSE), only the
      * blocks the batch touched (PSS_UPDATE_TOUCHED), or chosen from M and the
@@ -165,9 +169,10 @@ typedef enum {
      * state, any R; needs chunks that tile the rows (Z = 32, d a multiple of
      * 32, 16-byte aligned upstream gradient).  Other chunk shapes are grouped
      * within segments too, with the distinct locations counted, where R <=
-     * 2^22, the update is the dense one, the batch is one that PSS_PATH_AUTO
-     * would sort, and L is 4, 8 or 16 (chunks that tile the rows) or 32 to 128;
-     * else the global sort runs.
+     * 2^22, the update is the dense one, L is 4, 8 or 16 (chunks that tile the
+     * rows) or 32 to 128, and the batch adds at least 3,500,000 elements (L = 4,
+     * or fp32 accumulation: PSS_PATH_AUTO's 5,000,000 or 10,000,000); else the
+     * global sort runs.
      * PSS_SORT_AUTO (default): where the local sort is served, local if R >
      * 2^22 or the batch has at most PSS_SORT_LOCAL_MAX_PAIRS_PER_START pairs
      * per block start; local with a count of the distinct locations above

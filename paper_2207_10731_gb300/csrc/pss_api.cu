@@ -411,30 +411,18 @@ bool use_touched(const pss_handle* h, int64_t pairs) {
 
 // The sorted path holds bucket indices in 32 bits, 0xffffffff marking a bad
 // id: it needs R < kSortedMaxR, the bound below which the forward emits 32-bit
-// buckets at all.  AUTO takes the sorted path when the batch adds at least
-// auto_sorted_min_adds elements (pairs * L), the atomic path below: the
-// atomic path's one kernel wins small batches, the sorted path's sort and
-// reduce win large ones at every M from 2^18 to 2^33, Zipf or uniform ids.
-// Measured on GB300 (us of a whole step, atomic against sorted with the local
-// sort):
-//   L = 32, Criteo-TB shape, M = 2^18: 3.4M adds 38 / 27, 4.7M adds 40 / 29
-//   L = 16, Criteo-Kaggle shape, M = 2^20: 3.4M adds 52 / 42, 6.8M adds 94 / 49,
-//     13.6M adds 211 / 66
-//   L = 8, micro-benchmark shape, M = 2^18: 5.0M adds 71 / 43, 34M adds 261 / 157
-//   L = 64, 16.6M adds 127 / 62
-// (3.4M adds stay atomic as they were).  Without the local sort (run-to-run
-// identical bits, a forced global sort, shorter or untiled blocks) the sorted
-// path starts at 5M adds with blocks of 32 and more, 10M below; the fp32
-// atomic path is faster than the fp64 one and keeps those thresholds too.
+// buckets at all.
 constexpr int64_t kSortedMaxR = int64_t(0xffffffffLL);
 
-int64_t auto_sorted_min_adds(const pss_handle* h) {
-    const DevParams& p = h->dp;
-    const bool local = h->sort_scope != PSS_SORT_GLOBAL && !h->deterministic &&
-                       h->accum == PSS_ACCUM_F64 &&
-                       ((p.Z == 32 && p.d % 32 == 0) ||
-                        (p.L >= 8 && local_reduce_ok(p) && (int64_t)p.R <= kCountSortMaxR));
-    return local ? 3500000 : p.L >= 32 ? 5000000 : 10000000;
+// AUTO takes the sorted path when the batch adds at least this many elements
+// (pairs * L), the atomic path below: the atomic path's one kernel wins small
+// batches, the sorted path's sort and reduce win large ones at every M from 2^18
+// to 2^33, Zipf or uniform ids.
+int64_t auto_sorted_min_adds(const pss_handle* h) { return h->dp.L >= 32 ? 5000000 : 10000000; }
+
+// The least adds of a local sort of chunks that the staged reduce does not take.
+int64_t local_min_adds(const pss_handle* h) {
+    return h->dp.L >= 8 && h->accum == PSS_ACCUM_F64 ? 3500000 : auto_sorted_min_adds(h);
 }
 
 bool sorted_supported(const pss_handle* h, int64_t nnz, int64_t B) {
@@ -452,10 +440,82 @@ bool use_radix(const pss_handle* h) {
     return h->deterministic || (int64_t)h->dp.R > kCountSortMaxR;
 }
 
-bool want_sorted(const pss_handle* h, int64_t npairs) {
+// Bags of several ids: the sorted path reads a bag's gradient row once per id.
+bool rows_reread(const pss_handle* h, int64_t nnz, int64_t B) { return nnz > h->dp.T * B; }
+
+// How the sorted path groups the pairs (PSS_OPT_SORT_SCOPE): within segments,
+// with or without a count of the distinct buckets, or all of them.
+enum LocalSort { kLocalNo, kLocalUncounted, kLocalCounted };
+
+// The local sort saves the global sort's per-bucket counters and atomics but
+// leaves one run per bucket and segment, each an fp64 reduction of a chunk
+// into g.  Measured on GB300 (us of sort + reduce, global against local, with
+// the count of distinct buckets where AUTO makes it):
+//   one id per bag: 0.1M pairs over 65K starts 36 / 33 (whole step), 6.8M over
+//   65K, 262K, 625K, 1M starts 271 / 238, 281 / 234, 285 / 239, 291 / 243;
+//   1.06M over 625K 66 / 48; 2^24 starts: radix 343 / 110 with the marking
+//   several ids per bag (Zipf 1.05, Zipf 1.2), by pairs per start:
+//   16: 476 / 465, 424 / 377     27 (Zipf 1.2): 414 / 377
+//   33: 465 / 468, 426 / 380     65: 449 / 459, 413 / 374
+//   130: 430 / 454, 386 / 367
+// The gradient of bags of several ids comes from L2, so runs cost more there
+// and the global sort's few runs win from about 30 pairs per start on.
+constexpr int64_t kLocalMaxRereadPairsPerStart = 30;
+
+LocalSort use_local_sort(const pss_handle* h, int64_t nnz, int64_t B, bool touch,
+                         const float* dgrad) {
+    const int64_t R = (int64_t)h->dp.R, npairs = nnz * (int64_t)h->dp.J;
+    if (h->deterministic || h->sort_scope == PSS_SORT_GLOBAL) return kLocalNo;
+    if (!local_sort_ok(h->dp, dgrad)) {
+        // other chunk shapes: always counted, in batches of local_min_adds on
+        // (smaller ones leave the local sort's CTAs idle).  Measured on GB300,
+        // us of a whole step, global against local: micro-benchmark shape, M =
+        // 2^21, Z = 4, 8, 16, 64: 413 / 284, 230 / 154, 169 / 117, 122 / 110;
+        // Criteo-Kaggle shape, batch 32768: 136 / 66
+        return local_reduce_ok(h->dp) && !touch && R <= kCountSortMaxR &&
+                       npairs * (int64_t)h->dp.L >= local_min_adds(h)
+                   ? kLocalCounted
+                   : kLocalNo;
+    }
+    if (h->sort_scope == PSS_SORT_LOCAL || R > kCountSortMaxR ||
+        npairs <= (int64_t)PSS_SORT_LOCAL_MAX_PAIRS_PER_START * R)
+        return kLocalUncounted;
+    // (the touched list of a counted batch comes from the counting sort's scan)
+    if (touch || (rows_reread(h, nnz, B) && npairs > kLocalMaxRereadPairsPerStart * R))
+        return kLocalNo;
+    return kLocalCounted;
+}
+
+// Batches below AUTO's threshold that a local sort serves and whose reduce sums
+// every contribution in fp64, as the atomic path does (other sorted batches round
+// a run to fp32, see Sum32): AUTO sorts them from this many adds on.  The rule
+// asks what the backward will ask: `touch` as the update will have it, and the
+// upstream gradient's alignment (null: not known yet, taken as aligned).
+// Measured on GB300 (us of a whole Adagrad step, atomic against sorted; in brackets
+// with the runs summed in fp32):
+//   L = 16, Criteo-Kaggle shape, M = 2^20: 3.5M adds 52 / 39 (36), 6.7M 94 / 47
+//     (42), 10M 144 / 61 (52); M = 2^22, 6.7M 110 / 62
+//   L = 16 and 8, d = 128, M = 2.5M: 6.7M adds 76 / 50 (48), 81 / 56 (54)
+//   L = 32, Criteo-TB shape: 3.7M adds 45 / 38 (35), 4.7M 47 / 40 (36); M = 2^18,
+//     4.7M 37 / 31 (27)
+// (below 3.5M adds the sorted path was not measured with these sums).
+constexpr int64_t kAutoEarlyAdds = 3500000;
+bool auto_early(const pss_handle* h, int64_t nnz, int64_t B, const float* dgrad) {
+    const int64_t npairs = nnz * (int64_t)h->dp.J;
+    return npairs * (int64_t)h->dp.L >= kAutoEarlyAdds && h->accum == PSS_ACCUM_F64 &&
+           h->dp.L >= 8 && local_sums64_ok(h->dp, dgrad) &&
+           use_local_sort(h, nnz, B, use_touched(h, npairs), dgrad) != kLocalNo;
+}
+
+// The batch's contributions are summed in fp64 although it is sorted.
+bool sums64(const pss_handle* h, int64_t npairs) {
+    return h->path != PSS_PATH_SORTED && npairs * (int64_t)h->dp.L < auto_sorted_min_adds(h);
+}
+
+bool want_sorted(const pss_handle* h, int64_t nnz, int64_t B, const float* dgrad) {
     if (h->path == PSS_PATH_SORTED) return true;
     if (h->path == PSS_PATH_ATOMIC) return false;
-    return npairs * (int64_t)h->dp.L >= auto_sorted_min_adds(h);
+    return !sums64(h, nnz * (int64_t)h->dp.J) || auto_early(h, nnz, B, dgrad);
 }
 
 pss_status ensure_sorted(pss_handle* h, int64_t nnz, cudaStream_t st) {
@@ -800,7 +860,7 @@ pss_status pss_forward(pss_handle* h, const int64_t* indices, int64_t nnz, const
         dout = static_cast<float*>(h->st_out.ptr);
     }
     const bool emit =
-        nbags > 0 && want_sorted(h, nnz * (int64_t)h->dp.J) && sorted_supported(h, nnz, B);
+        nbags > 0 && want_sorted(h, nnz, B, nullptr) && sorted_supported(h, nnz, B);
     if (emit && (rc = ensure_sorted(h, nnz, st)) != PSS_OK) return rc;
     const int chunks = (host_out && nout * sizeof(float) >= kChunkedOutputBytes &&
                         B >= kForwardChunks && is_pinned_host_ptr(out))
@@ -861,51 +921,6 @@ static pss_status scatter_into(pss_handle* h, const float* dgrad, float scale, f
     return cuda_status(launch_scatter(h->dp, lay, h->last_idx, h->last_nnz,
                                       h->last_off, h->last_B, dgrad, scale, target,
                                       touch ? &h->touched : nullptr, h->err, h->sm_count, st));
-}
-
-// Bags of several ids: the sorted path reads a bag's gradient row once per id.
-static bool rows_reread(const pss_handle* h) { return h->last_nnz > h->dp.T * h->last_B; }
-
-// How the sorted path groups the pairs (PSS_OPT_SORT_SCOPE): within segments,
-// with or without a count of the distinct buckets, or all of them.
-enum LocalSort { kLocalNo, kLocalUncounted, kLocalCounted };
-
-// The local sort saves the global sort's per-bucket counters and atomics but
-// leaves one run per bucket and segment, each an fp64 reduction of a chunk
-// into g.  Measured on GB300 (us of sort + reduce, global against local, with
-// the count of distinct buckets where AUTO makes it):
-//   one id per bag: 0.1M pairs over 65K starts 36 / 33 (whole step), 6.8M over
-//   65K, 262K, 625K, 1M starts 271 / 238, 281 / 234, 285 / 239, 291 / 243;
-//   1.06M over 625K 66 / 48; 2^24 starts: radix 343 / 110 with the marking
-//   several ids per bag (Zipf 1.05, Zipf 1.2), by pairs per start:
-//   16: 476 / 465, 424 / 377     27 (Zipf 1.2): 414 / 377
-//   33: 465 / 468, 426 / 380     65: 449 / 459, 413 / 374
-//   130: 430 / 454, 386 / 367
-// The gradient of bags of several ids comes from L2, so runs cost more there
-// and the global sort's few runs win from about 30 pairs per start on.
-constexpr int64_t kLocalMaxRereadPairsPerStart = 30;
-
-static LocalSort use_local_sort(const pss_handle* h, int64_t npairs, bool touch,
-                                const float* dgrad) {
-    const int64_t R = (int64_t)h->dp.R;
-    if (h->deterministic || h->sort_scope == PSS_SORT_GLOBAL) return kLocalNo;
-    if (!local_sort_ok(h->dp, dgrad)) {
-        // other chunk shapes: always counted, in batches that AUTO would sort
-        // (smaller ones leave the local sort's CTAs idle).  Measured on GB300,
-        // us of a whole step, global against local: micro-benchmark shape, M =
-        // 2^21, Z = 4, 8, 16, 64: 413 / 284, 230 / 154, 169 / 117, 122 / 110;
-        // Criteo-Kaggle shape, batch 32768: 136 / 66
-        return local_reduce_ok(h->dp) && !touch && R <= kCountSortMaxR &&
-                       npairs * (int64_t)h->dp.L >= auto_sorted_min_adds(h)
-                   ? kLocalCounted
-                   : kLocalNo;
-    }
-    if (h->sort_scope == PSS_SORT_LOCAL || R > kCountSortMaxR ||
-        npairs <= (int64_t)PSS_SORT_LOCAL_MAX_PAIRS_PER_START * R)
-        return kLocalUncounted;
-    // (the touched list of a counted batch comes from the counting sort's scan)
-    if (touch || (rows_reread(h) && npairs > kLocalMaxRereadPairsPerStart * R)) return kLocalNo;
-    return kLocalCounted;
 }
 
 // The byte per bucket of a local sort that counts (zero between sorts: zeroed
@@ -983,7 +998,7 @@ static pss_status sorted_window(pss_handle* h, const float* dgrad, bool staged, 
     {
         LaunchScope ls(h, PSS_K_REDUCE, st, 2);
         const WindowSink ws{gexp, h->sb.bnd};
-        PSS_TRY(launch_window_reduce(h->sb, npairs, dgrad, h->dp, ws, rows_reread(h),
+        PSS_TRY(launch_window_reduce(h->sb, npairs, dgrad, h->dp, ws, rows_reread(h, h->last_nnz, h->last_B),
                                      h->sm_count, st));
     }
     return copy_stats(h, st);
@@ -1003,7 +1018,7 @@ static pss_status sorted_into64(pss_handle* h, const float* dgrad, bool staged, 
                                 cudaStream_t st) {
     const int64_t npairs = h->last_nnz * (int64_t)h->dp.J;
     if (h->dp.T * h->last_B == 0 || npairs == 0) return PSS_OK;
-    const LocalSort local = use_local_sort(h, npairs, touch, dgrad);
+    const LocalSort local = use_local_sort(h, h->last_nnz, h->last_B, touch, dgrad);
     pss_status rc0 = sort_pairs(h, touch, local, st);
     if (rc0 != PSS_OK) return rc0;
     // the sort above needs only the forward's buckets: a host gradient's copy
@@ -1013,7 +1028,8 @@ static pss_status sorted_into64(pss_handle* h, const float* dgrad, bool staged, 
     {
         LaunchScope ls(h, PSS_K_REDUCE, st);
         PSS_TRY(launch_sorted_reduce(h->sb, npairs, dgrad, h->dp, h->g64, local != kLocalNo,
-                                     local == kLocalNo && use_radix(h), rows_reread(h),
+                                     local == kLocalNo && use_radix(h), rows_reread(h, h->last_nnz, h->last_B),
+                                     sums64(h, npairs),
                                      local == kLocalCounted ? h->sb.seen : nullptr, h->sm_count,
                                      st));
     }
@@ -1038,7 +1054,7 @@ pss_status pss_backward_update(pss_handle* h, const float* grad_out, float lr, p
     if (rc != PSS_OK) return rc;
     const int64_t pairs = h->last_nnz * (int64_t)h->dp.J;
     const bool ada = h->opt == PSS_ADAGRAD;
-    const bool sorted = h->batch_emitted && want_sorted(h, h->last_nnz * (int64_t)h->dp.J);
+    const bool sorted = h->batch_emitted && want_sorted(h, h->last_nnz, h->last_B, dg);
     h->last_path = sorted ? PSS_PATH_SORTED : PSS_PATH_ATOMIC;
     if (sorted && h->deterministic && !h->circ && window_reduce_ok(h->dp, dg)) {
         // each element's gradient stored once into the fp32 buffer, then the
@@ -1146,7 +1162,7 @@ pss_status pss_backward_grad(pss_handle* h, const float* grad_out, float* grad, 
     bool staged = false;
     pss_status rc = stage_grad(h, grad_out, (size_t)nbags * (size_t)h->dp.d, st, &dg, &staged);
     if (rc != PSS_OK) return rc;
-    const bool sorted = h->batch_emitted && want_sorted(h, h->last_nnz * (int64_t)h->dp.J);
+    const bool sorted = h->batch_emitted && want_sorted(h, h->last_nnz, h->last_B, dg);
     h->last_path = sorted ? PSS_PATH_SORTED : PSS_PATH_ATOMIC;
     if (sorted && h->deterministic && !h->circ && window_reduce_ok(h->dp, dg)) {
         PSS_TRY(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)h->dp.M, st));

@@ -128,6 +128,8 @@ int64_t local_segments(int64_t npairs);
 bool local_sort_ok(const DevParams& p, const float* gout);
 // Other chunk shapes whose reduce takes the local layout.
 bool local_reduce_ok(const DevParams& p);
+// The shapes whose local reduce can also sum every contribution in fp64.
+bool local_sums64_ok(const DevParams& p, const float* gout);
 // With `touched`, also the touched bitmap and list of the buckets.
 cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
                               const Touched* touched, int sm_count, cudaStream_t st);
@@ -140,10 +142,13 @@ cudaError_t launch_count_seen(const SortedBuffers& sb, int64_t npairs, int64_t R
 // reduce counts the distinct buckets into stats[1] (the radix sort's entries;
 // the counting sort's scan counts them itself).  `reread`: the gradient's rows
 // are read several times (bags of several ids), so they are kept in L2.  `seen`
-// (local only, may be null): the buckets with entries are marked there.
+// (local only, may be null): the buckets with entries are marked there.  `sums64`
+// (local_sums64_ok): every contribution is summed in fp64, else a run in fp32 with
+// compensation.
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
-                                 bool reread, uint8_t* seen, int sm_count, cudaStream_t st);
+                                 bool reread, bool sums64, uint8_t* seen, int sm_count,
+                                 cudaStream_t st);
 // Window reduce (see pss_sorted.cu): run sums go into each task's sliding
 // element window; every element's gradient is stored once into gexp (fp32,
 // zero where the batch adds nothing; the caller zero-fills it), in a fixed

@@ -26,6 +26,7 @@
 // blocks.
 // The optimizer pass over g follows (pss_kernels.cu).
 #include <climits>
+#include <type_traits>
 
 #include "pss_device.cuh"
 #include "pss_internal.h"
@@ -1159,6 +1160,38 @@ k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
     if (!LOCAL && count_runs && lane == 0 && nstart) atomicAdd(stats + 1, (unsigned long long)nstart);
 }
 
+// The sum of one element over a run.  Sum32: fp32 with compensation, eight values
+// that continue the run as a tree first.  Sum64: fp64, every value widened and
+// added, as the atomic path does: for the batches that AUTO sorts only because
+// the sorted path is faster, so that they keep the atomic path's sums (the
+// rounding of a run to fp32 made the gradient's rms error 1.6 to 1.9 times as
+// large, and a run of an infinity and another value a NaN).
+struct Sum32 {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float v) { kahan_add(s, c, v); }
+    __device__ __forceinline__ void start(float v) {
+        s = c = 0.f;
+        add(v);
+    }
+    __device__ __forceinline__ void add8(const float (&v)[8]) {
+        const float a = (v[0] + v[1]) + (v[2] + v[3]);
+        const float b = (v[4] + v[5]) + (v[6] + v[7]);
+        add(a + b);
+    }
+    __device__ __forceinline__ double value() const { return widen(s); }
+};
+struct Sum64 {
+    double s = 0.0;
+    __device__ __forceinline__ void add(float v) { s += widen(v); }
+    __device__ __forceinline__ void start(float v) { s = widen(v); }
+    __device__ __forceinline__ void add8(const float (&v)[8]) {
+        const double a = (widen(v[0]) + widen(v[1])) + (widen(v[2]) + widen(v[3]));
+        const double b = (widen(v[4]) + widen(v[5])) + (widen(v[6]) + widen(v[7]));
+        s += a + b;
+    }
+    __device__ __forceinline__ double value() const { return s; }
+};
+
 // Reduce of a local sort's short chunks (L = 4, 8 or 16 elements that tile the
 // rows): groups of L lanes, lane z of a group on element z, each group summing
 // kGS consecutive entries of its own (compensated) and adding every run's sum
@@ -1173,7 +1206,7 @@ k_warp_range_reduce(const unsigned long long* __restrict__ sorted_e,
 constexpr int kGS = 64;   // entries per group
 constexpr int kGU = 8;    // chunks in flight per group
 
-template <int LOG2L, bool SG>
+template <int LOG2L, bool SG, typename Sum>
 __global__ void __launch_bounds__(kThreads)
 k_group_reduce(const unsigned long long* __restrict__ sorted_e, int64_t npairs,
                const uint32_t* __restrict__ segn, const float* __restrict__ gout, uint32_t G,
@@ -1204,7 +1237,7 @@ k_group_reduce(const unsigned long long* __restrict__ sorted_e, int64_t npairs,
     const float* gz = gout + z;
     double* const gl = g + z;
     uint32_t cur = (uint32_t)(ent[0] >> 32);
-    float sum = 0.f, comp = 0.f;
+    Sum sum;
     const int steps = n < kGS ? n : kGS;      // of the first group, the longest
     for (int i0 = 0; i0 < steps; i0 += kGU) {
         uint32_t x[kGU];
@@ -1221,14 +1254,15 @@ k_group_reduce(const unsigned long long* __restrict__ sorted_e, int64_t npairs,
 #pragma unroll
         for (int u = 0; u < kGU; ++u) {
             if (x[u] != cur) {
-                if (cur != kBad) red_add_f64(gl + (uint64_t)cur * G, widen(sum));
+                if (cur != kBad) red_add_f64(gl + (uint64_t)cur * G, sum.value());
                 cur = x[u];
-                sum = comp = 0.f;
+                sum.start(v[u]);
+            } else {
+                sum.add(v[u]);
             }
-            kahan_add(sum, comp, v[u]);
         }
     }
-    if (cur != kBad) red_add_f64(gl + (uint64_t)cur * G, widen(sum));
+    if (cur != kBad) red_add_f64(gl + (uint64_t)cur * G, sum.value());
 }
 
 // Reduce for 32-element chunks that tile the rows (Z = 32 dividing d).  Each
@@ -1299,7 +1333,7 @@ constexpr int kSinkOnce = 1;
 
 // LOCAL: the segment-local layout (k_sort_local): segment s holds segn[s] valid
 // entries from s*kLS on; otherwise one sorted run of stats[0] valid entries.
-template <int SINK, bool LOCAL, bool SG>
+template <int SINK, bool LOCAL, bool SG, typename Sum>
 __global__ void __launch_bounds__(kThreads, 4)
 k_async_reduce(const unsigned long long* __restrict__ sorted_e,
                unsigned long long* __restrict__ stats, int64_t npairs, int64_t per,
@@ -1361,7 +1395,8 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
     uint32_t cur = __shfl_sync(0xffffffffu, x0, 0);            // bucket of the open run
     uint32_t xlast = cur;                                      // last bucket of the block before
     uint32_t nstart = 0;   // distinct buckets: entries whose bucket differs from the one before
-    float sum = 0.f, comp = 0.f;
+    Sum sum;
+    static_assert(SINK == kSinkF64 || std::is_same<Sum, Sum32>::value, "the window adds in fp32");
     // the entry before the range: the window's head boundary, and whether the
     // range's first bucket counts as distinct
     uint32_t xprev = kBad;
@@ -1402,8 +1437,8 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
     double* const glane = g + lane;
     auto flush = [&]() {
         if (cur != kBad) {
-            if (SINK == kSinkF64) {
-                red_add_f64(glane + (uint64_t)cur * G, widen(sum));
+            if constexpr (SINK == kSinkF64) {
+                red_add_f64(glane + (uint64_t)cur * G, sum.value());
             } else {
                 const uint32_t dx = cur - wx;         // buckets ascend
                 if (dx != 0u) {
@@ -1418,10 +1453,9 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
                     wx = cur;
                     wb = (int64_t)cur * G;
                 }
-                kahan_add(acc, accc, sum - comp);
+                kahan_add(acc, accc, sum.s - sum.c);
             }
         }
-        sum = comp = 0.f;
     };
 
     for (int k = 0; k < nblk; ++k) {
@@ -1460,17 +1494,17 @@ k_async_reduce(const unsigned long long* __restrict__ sorted_e,
             }
             const uint32_t m = (heads >> (s * kAS)) & ((1u << kAS) - 1u);
             if (m == 0u) {
-                const float a = (v[0] + v[1]) + (v[2] + v[3]);
-                const float b = (v[4] + v[5]) + (v[6] + v[7]);
-                kahan_add(sum, comp, a + b);
+                sum.add8(v);
             } else {
 #pragma unroll
                 for (int i = 0; i < kAS; ++i) {
                     if (m & (1u << i)) {
                         flush();
                         cur = __shfl_sync(0xffffffffu, x0, s * kAS + i);
+                        sum.start(v[i]);
+                    } else {
+                        sum.add(v[i]);
                     }
-                    kahan_add(sum, comp, v[i]);
                 }
             }
         }
@@ -1614,8 +1648,11 @@ cudaError_t warp_reduce_inst(const SortedBuffers& sb, int64_t npairs, const floa
 
 template <int LOG2L>
 cudaError_t group_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
-                         const DevParams& p, double* g, uint8_t* seen, cudaStream_t st) {
-    const auto kern = p.smask ? k_group_reduce<LOG2L, true> : k_group_reduce<LOG2L, false>;
+                         const DevParams& p, double* g, bool sums64, uint8_t* seen,
+                         cudaStream_t st) {
+    const auto kern =
+        sums64 ? (p.smask ? k_group_reduce<LOG2L, true, Sum64> : k_group_reduce<LOG2L, false, Sum64>)
+               : (p.smask ? k_group_reduce<LOG2L, true, Sum32> : k_group_reduce<LOG2L, false, Sum32>);
     const int64_t per = (int64_t)(32 >> LOG2L) * kGS * kWarps;   // entries per CTA
     return launch_k(kern, dim3((unsigned)((npairs + per - 1) / per)), dim3(kThreads), 0, st,
                     sb.sorted_e, npairs, sb.segn, gout, (uint32_t)p.G, g, seen);
@@ -1822,7 +1859,7 @@ int64_t window_records(int64_t npairs, int sm_count) {
 }
 
 // The staged reduce over `entries` sorted entries, one range per warp.
-template <int SINK, bool LOCAL>
+template <int SINK, bool LOCAL, typename Sum = Sum32>
 static cudaError_t staged_reduce(const SortedBuffers& sb, int64_t npairs, int64_t entries,
                                  const float* gout, bool reread, const DevParams& p, double* g,
                                  const WindowSink& ws, const uint32_t* segn, bool count_runs,
@@ -1830,7 +1867,8 @@ static cudaError_t staged_reduce(const SortedBuffers& sb, int64_t npairs, int64_
     const int64_t per = staged_per(entries, staged_ctas(SINK, LOCAL, reread), sm_count);
     const int64_t tasks = (entries + per - 1) / per;
     const int grid = (int)((tasks + kWarps - 1) / kWarps);
-    auto kern = p.smask ? k_async_reduce<SINK, LOCAL, true> : k_async_reduce<SINK, LOCAL, false>;
+    auto kern = p.smask ? k_async_reduce<SINK, LOCAL, true, Sum>
+                        : k_async_reduce<SINK, LOCAL, false, Sum>;
     return launch_k(kern, dim3(grid), dim3(kThreads), 0, st, sb.sorted_e, sb.stats, npairs, per,
                     gout, reread, (uint32_t)p.G, g, ws, segn, count_runs, seen);
 }
@@ -1855,6 +1893,10 @@ bool local_sort_ok(const DevParams& p, const float* gout) { return window_reduce
 
 bool local_reduce_ok(const DevParams& p) {
     return group_reduce_ok(p) || (p.L >= 32 && p.L <= 128);
+}
+
+bool local_sums64_ok(const DevParams& p, const float* gout) {
+    return window_reduce_ok(p, gout) || group_reduce_ok(p);
 }
 
 cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, uint32_t smask,
@@ -1885,10 +1927,16 @@ cudaError_t launch_count_seen(const SortedBuffers& sb, int64_t npairs, int64_t R
 
 cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const float* gout,
                                  const DevParams& p, double* g, bool local, bool count_runs,
-                                 bool reread, uint8_t* seen, int sm_count, cudaStream_t st) {
+                                 bool reread, bool sums64, uint8_t* seen, int sm_count,
+                                 cudaStream_t st) {
+    if (sums64 && !local_sums64_ok(p, gout)) return cudaErrorInvalidValue;
     if (local && !window_reduce_ok(p, gout) && !local_reduce_ok(p)) return cudaErrorInvalidValue;
     // 32-element chunks tiling the rows: asynchronous shared-memory staging
     if (window_reduce_ok(p, gout)) {
+        if (local && sums64)
+            return staged_reduce<kSinkF64, true, Sum64>(sb, npairs, local_segments(npairs) * kLS,
+                                                        gout, reread, p, g, WindowSink{}, sb.segn,
+                                                        false, seen, sm_count, st);
         if (local)
             return staged_reduce<kSinkF64, true>(sb, npairs, local_segments(npairs) * kLS, gout,
                                                  reread, p, g, WindowSink{}, sb.segn, false, seen,
@@ -1907,9 +1955,9 @@ cudaError_t launch_sorted_reduce(const SortedBuffers& sb, int64_t npairs, const 
 #undef PSS_WR
     }
     if (local) {
-        if (p.L == 4) return group_reduce<2>(sb, npairs, gout, p, g, seen, st);
-        if (p.L == 8) return group_reduce<3>(sb, npairs, gout, p, g, seen, st);
-        return group_reduce<4>(sb, npairs, gout, p, g, seen, st);
+        if (p.L == 4) return group_reduce<2>(sb, npairs, gout, p, g, sums64, seen, st);
+        if (p.L == 8) return group_reduce<3>(sb, npairs, gout, p, g, sums64, seen, st);
+        return group_reduce<4>(sb, npairs, gout, p, g, sums64, seen, st);
     }
     const bool vec = (p.Z % 4 == 0) && (p.d % 4 == 0) && (((uintptr_t)gout & 15u) == 0);
     const int vw = vec ? 4 : 1;
