@@ -195,8 +195,9 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {   // a - b = 
 }
 
 // Compensated sums of VW-wide columns: add(v) is kahan_add per element,
-// add4 the tree sum of four values first; merge adds another lane's sum (the
-// compensations are added plainly: their rounding is of second order).
+// add4 the tree sum of four values first; merge adds another lane's sum, and its
+// compensation the same way (added plainly, 32 groups' sums were off by 2% more:
+// rms 5.3e-8 against 5.2e-8).
 template <int VW>
 struct Sum;
 template <>
@@ -220,10 +221,11 @@ struct Sum<4> {
         const uint64_t t1 = __shfl_xor_sync(0xffffffffu, s1, o);
         const uint64_t d0 = __shfl_xor_sync(0xffffffffu, c0, o);
         const uint64_t d1 = __shfl_xor_sync(0xffffffffu, c1, o);
+        constexpr uint64_t kNeg = 0x8000000080000000ull;
         kahan(s0, c0, t0);
         kahan(s1, c1, t1);
-        c0 = add2(c0, d0);
-        c1 = add2(c1, d1);
+        kahan(s0, c0, d0 ^ kNeg);
+        kahan(s1, c1, d1 ^ kNeg);
     }
     __device__ __forceinline__ float4 value() const {
         float4 v;
@@ -242,7 +244,7 @@ struct Sum<1> {
         const float os = __shfl_xor_sync(0xffffffffu, s, o);
         const float oc = __shfl_xor_sync(0xffffffffu, c, o);
         kahan_add(s, c, os);
-        c += oc;
+        kahan_add(s, c, -oc);
     }
     __device__ __forceinline__ float value() const { return s - c; }
 };
