@@ -121,10 +121,14 @@ inline int ceil_log2(int v) {
 
 // CTAs of `threads` threads and `smem` bytes of dynamic shared memory that fit
 // on an SM at once; shared memory above the default 48 KB is allowed first (on
-// every call: it belongs to the context).  The answer is a constant of the
-// kernel and the device, and asking the runtime costs about as much as a
-// launch: each thread keeps what it was told.
-inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, int* per_sm) {
+// every call: it belongs to the context).  What is allowed is `smem_most`, the
+// kernel's largest size, the same in every call: the limit is shared by all host
+// threads, and one that launches a smaller size must not lower it between
+// another's call here and its launch.  The answer is a constant of the kernel
+// and the device, and asking the runtime costs about as much as a launch: each
+// thread keeps what it was told.
+inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, size_t smem_most,
+                                 int* per_sm) {
     struct Known {
         const void* kernel;
         size_t smem;
@@ -132,9 +136,10 @@ inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, i
     };
     constexpr int kKnown = 64;
     static thread_local Known known[kKnown] = {};
+    if (smem > smem_most) return cudaErrorInvalidValue;
     if (smem > 48 * 1024) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(
+            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_most);
         if (e != cudaSuccess) return e;
     }
     int dev = 0;
@@ -154,12 +159,13 @@ inline cudaError_t resident_ctas(const void* kernel, int threads, size_t smem, i
     return cudaSuccess;
 }
 
-// Grid of a grid-stride kernel: all CTAs that fit at once, capped by the work.
+// Grid of a grid-stride kernel: all CTAs that fit at once, capped by the work
+// (smem_most: see resident_ctas; 0 where smem is the kernel's only size).
 template <typename K>
-int grid_for(K kernel, int sm_count, int64_t work_blocks, size_t smem = 0) {
+int grid_for(K kernel, int sm_count, int64_t work_blocks, size_t smem = 0, size_t smem_most = 0) {
     int per_sm = 1;
-    if (resident_ctas(reinterpret_cast<const void*>(kernel), kThreads, smem, &per_sm) !=
-        cudaSuccess)
+    if (resident_ctas(reinterpret_cast<const void*>(kernel), kThreads, smem,
+                      smem_most ? smem_most : smem, &per_sm) != cudaSuccess)
         per_sm = 1;
     int64_t g = (int64_t)sm_count * per_sm;
     if (work_blocks < g) g = work_blocks;

@@ -1751,7 +1751,7 @@ cudaError_t radix_pass(const SortedBuffers& sb, const unsigned long long* in,
     const size_t smem = radix_down_smem(nd);
     int per_sm = 1;   // (allows the shared memory)
     e = resident_ctas(reinterpret_cast<const void*>(down), kRThreads, smem,
-                      &per_sm);
+                      radix_down_smem(kRMaxDigits), &per_sm);
     if (e != cudaSuccess) return e;
     return launch_k(down, dim3(ntiles), dim3(kRThreads), smem, st, Pairs(sb), in, out,
                     npairs, sb.stats, J, log2J, shift, bits, ntiles, per, sb.cnt, sb.dstart);
@@ -1908,7 +1908,7 @@ cudaError_t launch_sort_local(const SortedBuffers& sb, int64_t npairs, int J, ui
     const size_t smem = local_smem(touched != nullptr);
     int per_sm = 1;
     const cudaError_t e =
-        resident_ctas(reinterpret_cast<const void*>(kern), kLSThreads, smem, &per_sm);
+        resident_ctas(reinterpret_cast<const void*>(kern), kLSThreads, smem, smem, &per_sm);
     if (e != cudaSuccess) return e;
     const int64_t nseg = local_segments(npairs), most = (int64_t)sm_count * per_sm;
     return launch_k(kern, dim3((unsigned)(nseg < most ? nseg : most)), dim3(kLSThreads), smem, st,

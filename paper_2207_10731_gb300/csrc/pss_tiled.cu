@@ -844,12 +844,13 @@ k_scatter_tiled(DevParams p, const int64_t* __restrict__ idx, int64_t nnz,
     }
 }
 
+constexpr int kStageBytes = 16384;   // staged buckets of the scatter
+
 TileGeom tile_geom(const DevParams& p, const RowLayout& lay, int64_t B, size_t xbytes) {
     TileGeom g;
     const int ng = 32 >> lay.log2gs;
     g.tb = kWarps * ng * kBagsPerGroup;
-    const int stage_bytes = 16384;
-    g.qc = stage_bytes / (int)(xbytes * (size_t)p.J);
+    g.qc = kStageBytes / (int)(xbytes * (size_t)p.J);
     if (g.qc < 1) g.qc = 1;
     g.tiles_per_table = (int)((B + g.tb - 1) / g.tb);
     return g;
@@ -866,6 +867,11 @@ size_t tile_smem(const TileGeom& g, const DevParams& p, size_t xbytes) {
 // against table by table: M = 2^20 144 / 157 (an earlier kernel), 2^24 182 /
 // 178, 2^25 195 / 191, 2^26 211 / 199, 2^28 220 / 204.
 constexpr int64_t kByTableMinM = int64_t(1) << 24;
+
+// The largest of all shapes: 32 lane groups per warp (a chunk's buckets fit:
+// J <= 512).
+constexpr size_t kTileSmemMost =
+    sizeof(int64_t) * (kWarps * 32 * kBagsPerGroup + 1) + kStageBytes;
 
 template <int VW, int KC, typename XT, bool SG, int MODE>
 cudaError_t fwd_mode(const DevParams& p, const RowLayout& lay, const int64_t* idx, int64_t nnz,
@@ -908,7 +914,8 @@ cudaError_t sc_inst(const DevParams& p, const RowLayout& lay, const int64_t* idx
     const TileGeom tg = tile_geom(p, lay, B, sizeof(XT));
     const size_t smem = tile_smem(tg, p, sizeof(XT));
     const int64_t ntiles = (int64_t)p.T * tg.tiles_per_table;
-    const int grid = grid_for(k_scatter_tiled<VW, KC, XT, AT, TOUCH>, sm_count, ntiles, smem);
+    const int grid =
+        grid_for(k_scatter_tiled<VW, KC, XT, AT, TOUCH>, sm_count, ntiles, smem, kTileSmemMost);
     return launch_k(k_scatter_tiled<VW, KC, XT, AT, TOUCH>, dim3(grid), dim3(kThreads), smem, st, p,
                     idx, nnz, off, B, gout, scale, target, tc, err, lay.log2gs, tg);
 }
