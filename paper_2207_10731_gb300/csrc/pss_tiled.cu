@@ -556,46 +556,22 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
     for (int k = 0; k < KC; ++k) wz[k] = w + col.zs[k];
     const int J = p.J;
     const int64_t ostride = (int64_t)p.T * p.d;
-    const int tpt = fg.tiles_per_table;
     const int bag = lane & ((1 << fg.log2pw) - 1);   // this lane's bag of the tile
     const int j0 = lane >> fg.log2pw;                // its first chunk
     const int lpb = 32 >> fg.log2pw;                 // lanes per bag
 
-    // tiles of this warp: tile number = r * T + t, or t * tpt + r (below 2^30,
-    // checked by the launcher), advanced without divisions, and with it the
-    // place of the lane's bag in the offsets
-    const bool by_table = fg.by_table;
-    const int nwarps = (int)gridDim.x * kWarps;
-    const int inner = by_table ? tpt : p.T;
-    const int step_out = nwarps / inner, step_in = nwarps - step_out * inner;
-    const int step_t = by_table ? step_out : step_in, step_r = by_table ? step_in : step_out;
-    const int64_t step_o = (int64_t)step_t * B + (int64_t)step_r * wb;
-    const int64_t wrap_o = by_table ? B - (int64_t)tpt * wb : wb - (int64_t)p.T * B;
-    const int tile0 = (int)blockIdx.x * kWarps + warp, out0 = tile0 / inner;
-    int t = by_table ? out0 : tile0 - out0 * inner;
-    int r = by_table ? tile0 - out0 * inner : out0;
-    if (t >= p.T || r >= tpt) return;
+    // tiles of this warp, and the place of the lane's bag in the offsets
+    const TileWalk walk(gridDim.x * kWarps, (uint32_t)p.T, (uint32_t)fg.tiles_per_table, B, wb,
+                        fg.by_table);
+    uint32_t t, r;
+    walk.first(blockIdx.x * kWarps + warp, t, r);
+    if (!walk.inside(t, r)) return;
     const int64_t* po = off + (int64_t)t * B + b_lo + (int64_t)r * wb + bag;
     const int64_t nbags = b_hi - b_lo;
-    auto advance = [&](int& tt, int& rr) {
-        tt += step_t;
-        rr += step_r;
-        po += step_o;
-        if (by_table ? rr >= tpt : tt >= p.T) {
-            if (by_table) {
-                rr -= tpt;
-                ++tt;
-            } else {
-                tt -= p.T;
-                ++rr;
-            }
-            po += wrap_o;
-        }
-    };
     // offsets of this lane's bag of tile (tt, rr) at po: a zero-length bag past the end
-    auto load_offsets = [&](int tt, int rr, int64_t& q0, int64_t& q1) {
+    auto load_offsets = [&](uint32_t tt, uint32_t rr, int64_t& q0, int64_t& q1) {
         q0 = q1 = 0;
-        if (bag < wb && tt < p.T && (int64_t)rr * wb + bag < nbags) {
+        if (bag < wb && tt < walk.T && (int64_t)rr * wb + bag < nbags) {
             q0 = __ldg(po);
             q1 = __ldg(po + 1);
         }
@@ -607,17 +583,17 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
 
     int64_t q0, q1, q0n, q1n;
     load_offsets(t, r, q0, q1);
-    int t1 = t, r1 = r;
-    advance(t1, r1);
+    uint32_t t1 = t, r1 = r;
+    po += walk.advance(t1, r1);
     load_offsets(t1, r1, q0n, q1n);
     if (pair_x && warp == 0 && b_lo == 0) {   // (these loads arrive with the tile's offsets)
         const int64_t a = __ldg(off), b = __ldg(off + (int64_t)p.T * B);
         if (a > 0 || b < nnz) drop_unused(a, b, nnz, J, pair_x, lane);
     }
     int64_t id = load_id(q0, q1);
-    while (t < p.T && r < tpt) {
-        int t2 = t1, r2 = r1;
-        advance(t2, r2);
+    while (walk.inside(t, r)) {
+        uint32_t t2 = t1, r2 = r1;
+        po += walk.advance(t2, r2);
         const int64_t idn = load_id(q0n, q1n);
         int64_t q0m, q1m;
         load_offsets(t2, r2, q0m, q1m);
@@ -625,8 +601,8 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
         const int64_t b0 = b_lo + (int64_t)r * wb;
         const int nb = (int)((b_hi - b0) < wb ? (b_hi - b0) : wb);
         float* obase = out + b0 * ostride + (int64_t)t * p.d;
-        const uint32_t row0 = (uint32_t)b0 * (uint32_t)p.T + (uint32_t)t;
-        const uint64_t tJ = (uint64_t)(uint32_t)t * (uint32_t)J;
+        const uint32_t row0 = (uint32_t)b0 * (uint32_t)p.T + t;
+        const uint64_t tJ = (uint64_t)t * (uint32_t)J;
         const uint64_t card = (uint64_t)__ldg(p.cards + t);
         const bool has = q1 > q0;
         const unsigned odd = __ballot_sync(0xffffffffu, q0 < 0 || q1 < q0 || q1 > nnz);
@@ -890,8 +866,7 @@ cudaError_t fwd_mode(const DevParams& p, const RowLayout& lay, const int64_t* id
     while (fg.log2pi < 5 && (2 << fg.log2pi) * p.J <= kWarpPairs) ++fg.log2pi;
     const int64_t tpt = (rows + fg.wb - 1) / fg.wb;
     const int64_t ntiles = (int64_t)p.T * tpt;
-    // (room for the stride past the last tile)
-    if (ntiles >= ((int64_t)1 << 30)) return cudaErrorInvalidValue;
+    if (ntiles >= kMaxTiles) return cudaErrorInvalidValue;
     fg.tiles_per_table = (int)tpt;
     fg.by_table = p.M >= kByTableMinM;
     fg.TJ = (uint64_t)p.T * (uint64_t)p.J;

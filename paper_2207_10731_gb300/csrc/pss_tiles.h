@@ -1,7 +1,14 @@
-// How the forward cuts a batch into tiles: host rules without CUDA types.
+// How the forward cuts a batch into tiles and its warps walk them: without CUDA
+// types, so that a host compiler takes it too.
 #pragma once
 
 #include <cstdint>
+
+#ifdef __CUDACC__
+#define PSS_HD __host__ __device__ __forceinline__
+#else
+#define PSS_HD inline
+#endif
 
 namespace pss {
 
@@ -33,5 +40,47 @@ inline int tile_bags(int64_t T, int J, int log2gs, int64_t rows, int64_t warps) 
     }
     return best;
 }
+
+// The tiles (table t, range r of wb bags) of one warp: every nwarps-th in the order
+// of the bags (number r * T + t) or of the tables (t * tpt + r), reached without
+// divisions.  32-bit numbers, below kMaxTiles (unsigned: a step or two past the
+// last tile stay in range).
+constexpr int64_t kMaxTiles = int64_t(1) << 31;
+
+struct TileWalk {
+    uint32_t T, tpt;              // tables, tiles per table
+    uint32_t step_t, step_r;
+    int64_t step_o, wrap_o;       // the same as distances in the offsets
+    bool by_table;
+    PSS_HD TileWalk(uint32_t nwarps, uint32_t T_, uint32_t tpt_, int64_t B, int wb, bool by_table_)
+        : T(T_), tpt(tpt_), by_table(by_table_) {
+        const uint32_t inner = by_table ? tpt : T;
+        const uint32_t step_out = nwarps / inner, step_in = nwarps - step_out * inner;
+        step_t = by_table ? step_out : step_in;
+        step_r = by_table ? step_in : step_out;
+        step_o = (int64_t)step_t * B + (int64_t)step_r * wb;
+        wrap_o = by_table ? B - (int64_t)tpt * wb : wb - (int64_t)T * B;
+    }
+    PSS_HD void first(uint32_t tile, uint32_t& t, uint32_t& r) const {
+        const uint32_t inner = by_table ? tpt : T, out = tile / inner;
+        t = by_table ? out : tile - out * inner;
+        r = by_table ? tile - out * inner : out;
+    }
+    PSS_HD bool inside(uint32_t t, uint32_t r) const { return t < T && r < tpt; }
+    // To the next tile; returns the distance in the offsets.
+    PSS_HD int64_t advance(uint32_t& t, uint32_t& r) const {
+        t += step_t;
+        r += step_r;
+        if (by_table ? r < tpt : t < T) return step_o;
+        if (by_table) {
+            r -= tpt;
+            ++t;
+        } else {
+            t -= T;
+            ++r;
+        }
+        return step_o + wrap_o;
+    }
+};
 
 }  // namespace pss
