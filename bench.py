@@ -357,11 +357,19 @@ def _sort_desc(h, binding, args):
         return {}
     if args.deterministic:
         return {"sort": "stable radix sort of all pairs"}
-    if info["last_collision_rate"] < 0:
-        return {"sort": "segment-local: pairs grouped by location within 8192-pair segments"}
-    return {"sort": ("counting sort of all pairs" if info["R"] <= (1 << 22) else
-                     "radix sort of all pairs"),
-            "collision_rate": info["last_collision_rate"]}
+    # a local pass may report a collision rate too: the handle says which sort ran (one that
+    # cannot: a rate stands for a global sort, whose kind follows R)
+    if hasattr(h, "last_grouping"):
+        local = h.last_grouping() == binding.GROUPED_LOCAL
+        counting = h.last_grouping() == binding.GROUPED_COUNTING
+    else:
+        local = info["last_collision_rate"] < 0
+        counting = info["R"] <= (1 << 22)
+    desc = {"sort": ("segment-local: pairs grouped by location within 8192-pair segments" if local
+                     else "counting sort of all pairs" if counting else "radix sort of all pairs")}
+    if info["last_collision_rate"] >= 0:
+        desc["collision_rate"] = info["last_collision_rate"]
+    return desc
 
 
 def _config_extra(args, w):

@@ -318,6 +318,12 @@ pss_status pss_get_error(pss_handle* h, int64_t* first_bad_index, pss_stream str
 /* Fill *info (host). */
 pss_status pss_get_info(pss_handle* h, pss_info* info);
 
+/* How the last backward grouped the pairs (PSS_GROUPED_NONE: not at all, or no
+ * backward yet; PSS_OPT_SORT_SCOPE describes the sorts). */
+enum { PSS_GROUPED_NONE = 0, PSS_GROUPED_LOCAL = 1, PSS_GROUPED_COUNTING = 2,
+       PSS_GROUPED_RADIX = 3 };
+pss_status pss_get_last_grouping(pss_handle* h, int32_t* grouping);
+
 /*
  * Profiling (with PSS_OPT_PROFILE = 1): synchronise, then report for kernel id
  * `kernel` the number of launches and their summed device time in ms since the

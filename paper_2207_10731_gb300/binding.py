@@ -32,6 +32,7 @@ ACCUM_F64, ACCUM_F32 = 0, 1
 PATH_AUTO, PATH_ATOMIC, PATH_SORTED = 0, 1, 2
 UPDATE_AUTO, UPDATE_DENSE, UPDATE_TOUCHED = 0, 1, 2
 SORT_AUTO, SORT_GLOBAL, SORT_LOCAL = 0, 1, 2
+GROUPED_NONE, GROUPED_LOCAL, GROUPED_COUNTING, GROUPED_RADIX = 0, 1, 2, 3
 K_LOCATIONS, K_FORWARD, K_SCATTER, K_UPDATE, K_SORT, K_REDUCE, K_MISC = range(7)
 KERNEL_NAMES = ["locations", "forward", "scatter", "update", "sort", "reduce", "misc"]
 
@@ -41,7 +42,7 @@ EXPORTS = [
     "pss_set_state", "pss_compute_locations", "pss_forward", "pss_backward_update",
     "pss_backward_grad", "pss_set_option", "pss_get_option", "pss_get_error", "pss_get_info",
     "pss_get_profile", "pss_reset_profile", "pss_status_string", "pss_grad_noalloc",
-    "pss_check_convert", "pss_probe_l2",
+    "pss_check_convert", "pss_probe_l2", "pss_get_last_grouping",
 ]
 
 
@@ -94,6 +95,7 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
             "pss_get_option": [vp, i32, vp],
             "pss_get_error": [vp, vp, vp],
             "pss_get_info": [vp, vp],
+            "pss_get_last_grouping": [vp, vp],
             "pss_get_profile": [vp, i32, vp, vp],
             "pss_reset_profile": [vp],
             "pss_grad_noalloc": [vp, i32, i32, i64, i32, i32, u64, vp, i64, vp, i64, vp, vp, vp,
@@ -307,6 +309,12 @@ class PSS:
         inf = PSSInfo()
         _check(self._lib.pss_get_info(self._h, ctypes.byref(inf)), "pss_get_info")
         return {name: getattr(inf, name) for name, _ in PSSInfo._fields_}
+
+    def last_grouping(self) -> int:
+        """How the last backward grouped the pairs: GROUPED_NONE, _LOCAL, _COUNTING or _RADIX."""
+        v = ctypes.c_int32()
+        _check(self._lib.pss_get_last_grouping(self._h, ctypes.byref(v)), "pss_get_last_grouping")
+        return int(v.value)
 
     def profile(self, kernel: int):
         n, ms = ctypes.c_int64(), ctypes.c_double()

@@ -72,6 +72,7 @@ struct pss_handle {
     int64_t sort_scope = PSS_SORT_AUTO;         // PSS_OPT_SORT_SCOPE
     int64_t last_path = PSS_PATH_ATOMIC;
     int64_t last_update = 0;                    // pss_info.last_update
+    int32_t last_grouping = PSS_GROUPED_NONE;   // pss_get_last_grouping
     double last_collision = -1.0;
 
     Staging st_idx, st_off, st_out, st_grad, st_locs;
@@ -939,6 +940,9 @@ static pss_status sort_pairs(pss_handle* h, bool touch, LocalSort local, cudaStr
     const int64_t npairs = h->last_nnz * (int64_t)h->dp.J;
     h->sb.R = (uint32_t)h->dp.R;   // (below 2^32, and so are the rows: sorted_supported)
     h->sb.rows = (uint32_t)(h->dp.T * h->last_B);
+    h->last_grouping = local != kLocalNo ? PSS_GROUPED_LOCAL
+                       : use_radix(h)    ? PSS_GROUPED_RADIX
+                                         : PSS_GROUPED_COUNTING;
     poll_stats(h);
     if (local != kLocalNo) {
         // grouped within segments only: the distinct buckets are marked and
@@ -1056,6 +1060,7 @@ pss_status pss_backward_update(pss_handle* h, const float* grad_out, float lr, p
     const bool ada = h->opt == PSS_ADAGRAD;
     const bool sorted = h->batch_emitted && want_sorted(h, h->last_nnz, h->last_B, dg);
     h->last_path = sorted ? PSS_PATH_SORTED : PSS_PATH_ATOMIC;
+    h->last_grouping = PSS_GROUPED_NONE;
     if (sorted && h->deterministic && !h->circ && window_reduce_ok(h->dp, dg)) {
         // each element's gradient stored once into the fp32 buffer, then the
         // update pass (which returns the buffer to zero)
@@ -1164,6 +1169,7 @@ pss_status pss_backward_grad(pss_handle* h, const float* grad_out, float* grad, 
     if (rc != PSS_OK) return rc;
     const bool sorted = h->batch_emitted && want_sorted(h, h->last_nnz, h->last_B, dg);
     h->last_path = sorted ? PSS_PATH_SORTED : PSS_PATH_ATOMIC;
+    h->last_grouping = PSS_GROUPED_NONE;
     if (sorted && h->deterministic && !h->circ && window_reduce_ok(h->dp, dg)) {
         PSS_TRY(cudaMemsetAsync(grad, 0, sizeof(float) * (size_t)h->dp.M, st));
         if ((rc = sorted_window(h, dg, staged, false, grad, st)) != PSS_OK) return rc;
@@ -1315,6 +1321,12 @@ pss_status pss_get_info(pss_handle* h, pss_info* info) {
     info->last_path = h->last_path;
     info->last_update = h->last_update;
     info->last_collision_rate = h->last_collision;
+    return PSS_OK;
+}
+
+pss_status pss_get_last_grouping(pss_handle* h, int32_t* grouping) {
+    if (!h || !grouping) return PSS_ERR_INVALID_ARG;
+    *grouping = h->last_grouping;
     return PSS_OK;
 }
 
