@@ -151,7 +151,10 @@ def _stream_ptr(stream):
         return int(stream.cuda_stream)
     torch = _torch()
     if torch.cuda.is_initialized():
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:
+            pass   # torch's internals, which another version may lack
     return int(torch.cuda.current_stream().cuda_stream)
 
 
