@@ -267,11 +267,12 @@ pss_status grad_release(pss_handle* h, bool staged, cudaStream_t st) {
 }
 
 // The array (n == M values from the library's buffer `src`) to the caller.  A
-// kernel where both lie in this device's memory and fit in L2: it is launched
-// behind the kernel before it without a gap, and reads what the update left in
-// L2.  Measured on GB300 for 2.5M values: 3.6 us against 7.5 for the runtime's
-// copy, and 6 us less for a whole Criteo-TB step of 2048 rows.  Larger arrays
-// move at HBM rate either way (2^26 values: 82 us).
+// kernel where both lie in this device's memory, up to kCopyKernelMax values (source
+// and copy are 128 MB then, about the L2): it is launched behind the kernel before
+// it without a gap, and reads what the update left in L2.  Measured on GB300 for
+// 2.5M values: 3.6 us against 7.5 for the runtime's copy, and 6 us less for a whole
+// Criteo-TB step of 2048 rows.  Larger arrays move at HBM rate either way (2^26
+// values: 82 us).
 constexpr int64_t kCopyKernelMax = int64_t(1) << 24;
 pss_status copy_out(pss_handle* h, float* dst, const float* src, int64_t n, cudaStream_t st) {
     if (n <= kCopyKernelMax && ((uintptr_t)dst & 15u) == 0 && is_own_device_ptr(dst, h->device))
@@ -459,8 +460,11 @@ enum LocalSort { kLocalNo, kLocalUncounted, kLocalCounted };
 //   16: 476 / 465, 424 / 377     27 (Zipf 1.2): 414 / 377
 //   33: 465 / 468, 426 / 380     65: 449 / 459, 413 / 374
 //   130: 430 / 454, 386 / 367
-// The gradient of bags of several ids comes from L2, so runs cost more there
-// and the global sort's few runs win from about 30 pairs per start on.
+// The gradient of bags of several ids comes from L2, so runs cost more there: from
+// about 30 pairs per start on the global sort's few runs win by 1% to 6% with Zipf
+// 1.05 ids.  With the hotter ids of Zipf 1.2, whose repeats meet within a segment,
+// the local sort stays 5% to 11% faster up to 130; the rule does not see the ids,
+// and keeps the global sort there.
 constexpr int64_t kLocalMaxRereadPairsPerStart = 30;
 
 LocalSort use_local_sort(const pss_handle* h, int64_t nnz, int64_t B, bool touch,

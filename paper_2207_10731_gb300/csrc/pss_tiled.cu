@@ -529,8 +529,8 @@ __device__ __noinline__ void drop_tile(int64_t qa, int64_t qb, int64_t nnz, int 
 // own, and in tiles whose bags all hold one valid id a row costs one
 // shared-memory load, one multiply-add, one load and one store.  Tiles run
 // over the tables of a range of bags first, so that the rows that the GPU
-// writes at a time are one contiguous piece of the output (arrays beyond the
-// L2: over the bags of a table first, see kByTableMinM).
+// writes at a time are one contiguous piece of the output (large arrays: over
+// the bags of a table first, see kByTableMinM).
 template <int VW, int KC, typename XT, bool SG, int MODE>
 __global__ void __launch_bounds__(kThreads, fwd_min_ctas(VW, KC, MODE))
 k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ idx, int64_t nnz,
@@ -836,12 +836,14 @@ size_t tile_smem(const TileGeom& g, const DevParams& p, size_t xbytes) {
     return sizeof(int64_t) * (size_t)(g.tb + 1) + xbytes * (size_t)g.qc * (size_t)p.J;
 }
 
-// Arrays from this many elements on take their tiles table by table: beyond the
-// L2 the blocks of one table's hot ids stay in it better than those of all
-// tables at once; smaller arrays take them bag by bag, whose rows HBM writes
-// better.  Measured on GB300, us per serving forward of 65536 rows, bag by bag
-// against table by table: M = 2^20 144 / 157 (an earlier kernel), 2^24 182 /
-// 178, 2^25 195 / 191, 2^26 211 / 199, 2^28 220 / 204.
+// Arrays from this many elements on take their tiles table by table: the larger
+// the array, the better the blocks of one table's hot ids stay in the L2 than
+// those of all tables at once; smaller arrays take them bag by bag, whose rows HBM
+// writes better.  The line is where the two cross.  Measured on GB300, us per
+// serving forward, bag by bag against table by table: 65536 rows of one id (d =
+// 128) M = 2^20 143 / 150, 2^22 148 / 156, 2^23 161 / 164, 2^24 182 / 178, 2^25
+// 194 / 191, 2^26 208 / 199, 2^28 219 / 203; 16384 rows of 20 ids per bag (d = 64)
+// 2^22 211 / 211, 2^24 238 / 225, 2^26 254 / 231.
 constexpr int64_t kByTableMinM = int64_t(1) << 24;
 
 // The largest of all shapes: 32 lane groups per warp (a chunk's buckets fit:
