@@ -506,8 +506,9 @@ forward_bags(const DevParams& p, const FwdGeom& fg, const int64_t* __restrict__ 
 // and last offset, and one warp of every CTA calls this.
 __device__ __noinline__ void drop_unused(int64_t a, int64_t b, int64_t nnz, int J,
                                          uint32_t* __restrict__ pair_x, int lane) {
-    const int64_t head = (a < nnz ? a : nnz) * J;
-    const int64_t tail = (b < 0 ? 0 : b) * J;
+    // (malformed offsets are any 64-bit numbers: into [0, nnz] before a product)
+    const int64_t head = (a < 0 ? 0 : a < nnz ? a : nnz) * J;
+    const int64_t tail = (b < 0 ? 0 : b < nnz ? b : nnz) * J;
     const int64_t stride = (int64_t)gridDim.x * 32, k0 = (int64_t)blockIdx.x * 32 + lane;
     for (int64_t k = k0; k < head; k += stride) pair_x[k] = Invalid<uint32_t>::v;
     for (int64_t k = tail + k0; k < nnz * J; k += stride) pair_x[k] = Invalid<uint32_t>::v;
@@ -518,7 +519,7 @@ __device__ __noinline__ void drop_unused(int64_t a, int64_t b, int64_t nnz, int 
 __device__ __noinline__ void drop_tile(int64_t qa, int64_t qb, int64_t nnz, int J,
                                        uint32_t* __restrict__ pair_x, int lane) {
     constexpr int64_t kMost = 1 << 16;   // pairs
-    if (qa < 0 || qb > nnz || (qb - qa) * J > kMost) return;
+    if (qa < 0 || qb < qa || qb > nnz || (qb - qa) * J > kMost) return;
     for (int64_t k = qa * J + lane; k < qb * J; k += 32) pair_x[k] = Invalid<uint32_t>::v;
 }
 
@@ -578,7 +579,7 @@ k_forward_warp(const __grid_constant__ DevParams p, const int64_t* __restrict__ 
     };
     // the id of a bag that holds exactly one (offsets in range), else -1
     auto load_id = [&](int64_t q0, int64_t q1) -> int64_t {
-        return (q0 >= 0 && q1 == q0 + 1 && q1 <= nnz) ? __ldg(idx + q0) : -1;
+        return (q0 >= 0 && q0 < nnz && q1 == q0 + 1) ? __ldg(idx + q0) : -1;
     };
 
     int64_t q0, q1, q0n, q1n;

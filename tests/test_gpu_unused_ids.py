@@ -92,6 +92,18 @@ def test_malformed_offsets_stay_inside_the_buffers(sort):
         h.forward(gu.cuda(w.indices), gu.cuda(off), B)
         assert np.isfinite(gu.host(h.backward_grad(go))).all()
         assert h.get_error() == (binding.PSS_ERR_INDEX_RANGE, -2)
+    # numbers whose products and successors leave 64 bits
+    top = (1 << 63) - 1
+    for at, v in ((0, -(1 << 62)), (0, 1 << 62), (0, -top // 3), (-1, 1 << 62), (-1, -(1 << 62)),
+                  (-1, top // 3), (-1, top), (0, -top - 1), (96, 1 << 62), (96, -top // 3),
+                  (96, top), (101, -top - 1)):
+        h.forward(gu.cuda(w.indices), gu.cuda(with_(at, v)), B)
+        assert np.isfinite(gu.host(h.backward_grad(go))).all()
+        assert h.get_error() == (binding.PSS_ERR_INDEX_RANGE, -2)
+    off = w.offsets.copy()
+    off[50], off[51] = top, -top - 1
+    h.forward(gu.cuda(w.indices), gu.cuda(off), B)
+    assert h.get_error() == (binding.PSS_ERR_INDEX_RANGE, -2)
     # an offset inside a tile (of 4, 8, .. 32 bags): that tile's ids add nothing, all others do
     off = with_(5, w.offsets[5] - 100)
     h.forward(gu.cuda(w.indices), gu.cuda(off), B)
