@@ -359,7 +359,7 @@ k_sort_scatter(const Pairs pairs, int64_t npairs, int J, int log2J, uint32_t* __
 // What bounds it: the latency of a segment's phases (load, rank, scan, place,
 // write).  So the entries are placed in the counters' own shared memory once
 // every place is known, and two CTAs of 1024 threads share an SM.  Measured on
-// GB300: 41 us at the Criteo-TB shape (6.8M pairs), 9.2 us at the
+// GB300: 42 us at the Criteo-TB shape (6.8M pairs), 9.3 us at the
 // micro-benchmark's (1.06M), against 64 and 12.7 us with a hash table of keys
 // and counts (128 KB, one CTA per SM, a compare-and-swap per pair).
 constexpr int kLSLog2 = 13;
